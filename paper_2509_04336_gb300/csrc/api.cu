@@ -496,20 +496,27 @@ extern "C" int ns_walk_batch(ns_handle* h, int event, const double* live_u, int 
   T.done = 0;
   T.event = event;
   T.spec = E.cfg.spec_depth > 0 ? E.cfg.spec_depth : default_spec(h->precision);
+  T.spec_cap = E.cfg.spec_depth > 0 ? 0 : kSpecMax;
   watchdog_fields(h, T);
   cudaError_t e;
-  if ((e = cudaMemsetAsync(h->d_status + 1, 0, sizeof(int32_t) * 2, s)) != cudaSuccess) return cuda_fail(h, e, "status reset");
+  // the flow's timeout bit and the walks' watchdog bit: launch_walk_prepare clears both, but a
+  // flow's proposal table is made before it
+  const bool flow = walk_uses_flow(h, event);
+  if (flow && (e = cudaMemsetAsync(h->d_status + 1, 0, sizeof(int32_t) * 2, s)) != cudaSuccess)
+    return cuda_fail(h, e, "status reset");
   int fr = flow_attach(h, event, T, n, n_steps, &h->scratch_flow, s);
   if (fr) return fr;
-  // block -> (event, walker) maps, one task slot of the handle
-  int r = ensure_scratch(h, h->scratch_map, sizeof(int32_t) * 2 * (size_t)n + sizeof(WalkTask));
+  // one task slot of the handle, block -> (event, walker) maps, the survivors as float pairs
+  const size_t nu = (size_t)n * D, ns_ = (size_t)n_live_pts * D;
+  const size_t task_b = (sizeof(WalkTask) + 255) / 256 * 256, map_b = (sizeof(int32_t) * 2 * (size_t)n + 255) / 256 * 256;
+  int r = ensure_scratch(h, h->scratch_map, task_b + map_b + sizeof(float2) * ns_);
   if (r) return r;
   WalkTask* d_task = (WalkTask*)h->scratch_map.ptr;
-  int32_t* d_be = (int32_t*)((char*)h->scratch_map.ptr + sizeof(WalkTask));
+  int32_t* d_be = (int32_t*)((char*)h->scratch_map.ptr + task_b);
   int32_t* d_bl = d_be + n;
-  std::vector<int32_t> maps(2 * (size_t)n);
-  for (int j = 0; j < n; ++j) { maps[j] = 0; maps[n + j] = j; }
-  size_t nu = (size_t)n * D, ns_ = (size_t)n_live_pts * D;
+  float2* d_survf = (float2*)((char*)h->scratch_map.ptr + task_b + map_b);
+  T.survf = d_survf;
+  int32_t* clear = flow ? nullptr : h->d_status + 1;
   if (ptr_kind == NS_PTR_HOST) {
     if (!finite_array(live_u, (int)ns_) || !finite_array(u0, (int)nu)) return set_error(h, NS_ENONFINITE, "u not finite");
     size_t in_b = sizeof(double) * (ns_ + nu + n);
@@ -526,11 +533,10 @@ extern "C" int ns_walk_batch(ns_handle* h, int event, const double* live_u, int 
     T.surv = d_surv; T.u0 = d_u0; T.lnl0 = d_l0; T.u_out = d_uo; T.lnl_out = d_lo; T.n_acc = d_na; T.n_like = d_nl;
     if ((e = cudaMemcpyAsync(d_surv, live_u, sizeof(double) * ns_, cudaMemcpyHostToDevice, s)) ||
         (e = cudaMemcpyAsync(d_u0, u0, sizeof(double) * nu, cudaMemcpyHostToDevice, s)) ||
-        (e = cudaMemcpyAsync(d_l0, lnl0, sizeof(double) * n, cudaMemcpyHostToDevice, s)) ||
-        (e = cudaMemcpyAsync(d_task, &T, sizeof(T), cudaMemcpyHostToDevice, s)) ||
-        (e = cudaMemcpyAsync(d_be, maps.data(), sizeof(int32_t) * 2 * n, cudaMemcpyHostToDevice, s)))
+        (e = cudaMemcpyAsync(d_l0, lnl0, sizeof(double) * n, cudaMemcpyHostToDevice, s)))
       return cuda_fail(h, e, "H2D walk inputs");
-    if ((e = launch_walk(h->precision, h->waveform, E.n_det, h->d_events, d_task, d_be, d_bl, n, s, walk_extras(h, event))) != cudaSuccess)
+    if ((e = launch_walk_prepare(T, d_task, d_be, d_bl, d_survf, clear, ns_, s)) != cudaSuccess ||
+        (e = launch_walk(h->precision, h->waveform, E.n_det, h->d_events, d_task, d_be, d_bl, n, s, walk_extras(h, event))) != cudaSuccess)
       return cuda_fail(h, e, "walk launch");
     if ((e = cudaMemcpyAsync(u_out, d_uo, sizeof(double) * nu, cudaMemcpyDeviceToHost, s)) ||
         (e = cudaMemcpyAsync(lnl_out, d_lo, sizeof(double) * n, cudaMemcpyDeviceToHost, s)) ||
@@ -543,12 +549,8 @@ extern "C" int ns_walk_batch(ns_handle* h, int event, const double* live_u, int 
     return NS_OK;
   }
   T.surv = live_u; T.u0 = u0; T.lnl0 = lnl0; T.u_out = u_out; T.lnl_out = lnl_out; T.n_acc = n_accept; T.n_like = n_like;
-  // The task and the block maps go through the handle's scratch, ordered on the stream
-  // before the launch (a pageable-memory copy has consumed its source when it returns).
-  std::vector<char> stage((char*)&T, (char*)&T + sizeof(T));
-  stage.insert(stage.end(), (char*)maps.data(), (char*)maps.data() + sizeof(int32_t) * 2 * n);
-  if ((e = cudaMemcpyAsync(d_task, stage.data(), stage.size(), cudaMemcpyHostToDevice, s)))
-    return cuda_fail(h, e, "H2D walk task");
+  if ((e = launch_walk_prepare(T, d_task, d_be, d_bl, d_survf, clear, ns_, s)) != cudaSuccess)
+    return cuda_fail(h, e, "walk task launch");
   e = launch_walk(h->precision, h->waveform, E.n_det, h->d_events, d_task, d_be, d_bl, n, s, walk_extras(h, event));
   return e == cudaSuccess ? NS_OK : cuda_fail(h, e, "walk launch");
 }
@@ -561,10 +563,12 @@ void watchdog_fields(ns_handle* h, WalkTask& T) {
   T.budget_ns = h->budget_ns;
 }
 
-bool walk_extras(const ns_handle* h, int e) {
+bool walk_uses_flow(const ns_handle* h, int e) {
   const EventHost& E = h->events[e];
-  return E.dev.rb_nb > 0 || (E.flow.enabled && E.flow.p_flow > 0.0);
+  return E.flow.enabled && E.flow.p_flow > 0.0;
 }
+
+bool walk_extras(const ns_handle* h, int e) { return h->events[e].dev.rb_nb > 0 || walk_uses_flow(h, e); }
 
 bool walk_extras(const ns_handle* h) {
   for (int e = 0; e < (int)h->events.size(); ++e)

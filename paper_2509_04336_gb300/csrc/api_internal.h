@@ -128,6 +128,7 @@ int default_spec(int precision);
 int hrss_default_spec(int waveform);
 // Whether a walk of event e (of any event of the handle) uses flow proposals or the
 // relative-binning likelihood: launch_walk's extras.
+bool walk_uses_flow(const ns_handle* h, int e);
 bool walk_extras(const ns_handle* h, int e);
 bool walk_extras(const ns_handle* h);
 void nested_free(ns_handle* h);

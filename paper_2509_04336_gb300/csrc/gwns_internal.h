@@ -43,7 +43,7 @@ struct WalkTask {
   const double* flq;       // [n][f_stride]
   double p_flow;
   int32_t f_stride;
-  int32_t pad_;
+  int32_t spec_cap;        // largest depth a walker may adapt its own to (0: spec stays fixed)
   // hit-and-run slice sampling (HRSS) tasks: the lower Cholesky factor [D][D] of the
   // survivors' covariance; n_steps counts moves
   const double* chol;
@@ -74,6 +74,10 @@ cudaError_t launch_hrss(int precision, int waveform, int n_det, const EventDev* 
                         const int32_t* d_blk_task, const int32_t* d_blk_local, int n_blocks, cudaStream_t s);
 // Fills the FP64 path's angle table on the current device (before any FP64 likelihood runs).
 cudaError_t turn_table_upload(cudaStream_t s);
+// Writes a stand-alone walk's task and block maps (task 0, walker j on block j) and the float-pair
+// copy survf of the n_surv survivor coordinates T.surv; clears clear[0], clear[1] (if not null).
+cudaError_t launch_walk_prepare(const WalkTask& T, WalkTask* d_task, int32_t* d_blk_task, int32_t* d_blk_local,
+                                float2* d_survf, int32_t* clear, size_t n_surv, cudaStream_t s);
 // Block b walks walker blk_local[b] of task blk_task[b].  extras: some task of the launch uses
 // flow proposals or the relative-binning likelihood (false lets mode 2 run a walk kernel
 // compiled without those paths).

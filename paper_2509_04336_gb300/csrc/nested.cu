@@ -582,6 +582,7 @@ int nested_init(ns_handle* h) {
     std::memset(&T, 0, sizeof(T));
     T.surv = S.surv_u; T.survf = S.survf; T.u0 = S.w_u0; T.lnl0 = S.w_lnl0; T.u_out = S.w_uo; T.lnl_out = S.w_lo;
     T.n_acc = S.w_na; T.n_like = S.w_nl; T.n_bins = S.w_nb; T.n_spec = S.w_ns; T.spec = S.spec;
+    T.spec_cap = S.spec_auto ? S.spec_cap : 0;
     T.n_acc_flow = S.w_naf;
     T.lnl_star = -INFINITY; T.iteration = 0; T.walker_offset = 0;
     T.key0 = S.key0; T.key1 = S.key1; T.n_s = S.n_live - S.k; T.n = S.k; T.n_steps = S.n_steps;
@@ -679,7 +680,8 @@ int set_spec_cap(ns_handle* h, int cap) {
     cudaError_t err;
     if ((err = copy_on(h, &d->spec_cap, &cap, sizeof(int32_t), cudaMemcpyHostToDevice)) ||
         (err = copy_on(h, &d->spec, &spec, sizeof(int32_t), cudaMemcpyHostToDevice)) ||
-        (err = copy_on(h, &h->d_tasks[e].spec, &spec, sizeof(int32_t), cudaMemcpyHostToDevice)))
+        (err = copy_on(h, &h->d_tasks[e].spec, &spec, sizeof(int32_t), cudaMemcpyHostToDevice)) ||
+        (err = copy_on(h, &h->d_tasks[e].spec_cap, &cap, sizeof(int32_t), cudaMemcpyHostToDevice)))
       return cuda_fail(h, err, "speculation cap");
   }
   return NS_OK;
@@ -716,12 +718,15 @@ extern "C" int ns_step(ns_handle* h, int max_batches, ns_progress* progress) {
     // moves time.
     int64_t it_now = h->host_ns.empty() ? 0 : h->host_ns[0].iteration;
     // First cap, from the cost structure once a batch has run: a proposal of fewer than ~1k
-    // active bins (with relative binning: edges plus exact-range bins) is a short likelihood whose rounds are dominated by fixed costs (largest
-    // cap); a longer one costs a full evaluation per speculative proposal (small cap).
+    // active bins (with relative binning: edges plus exact-range bins) is a short likelihood whose
+    // rounds are dominated by fixed costs (largest cap); a longer one costs a full evaluation per
+    // speculative proposal (small cap) -- except in the float-float IMRPhenomD-form walk, whose
+    // rounds end at their first acceptance and evaluate nothing in vain (largest cap).
     if (h->tune && !h->tune_guessed && it_now >= 1) {
       double bins = 0.0, evals = 0.0;
       for (auto& S : h->host_ns) { bins += (double)S.n_bins_eval; evals += (double)S.n_spec_eval; }
-      const bool short_lik = evals > 0.0 && bins < 1024.0 * evals;
+      const bool short_lik = (evals > 0.0 && bins < 1024.0 * evals) ||
+                             (h->precision == NS_PREC_MIXED_FF && h->waveform == NS_WAVEFORM_PHENOMD_FORM);
       const int cap = h->precision == 0 ? (short_lik ? 8 : 2) : (short_lik ? 32 : 4);
       if ((r = set_spec_cap(h, cap))) return r;
       h->tune_best = cap;
@@ -970,7 +975,9 @@ extern "C" int ns_state_load(ns_handle* h, const char* path) {
     std::memcpy(&S, &R.S, offsetof(NsState, live_u));
     S.dead_cap = E.ns.dead_cap;
     WalkTask* dt = h->d_tasks + e;
+    const int32_t task_cap = S.spec_auto ? S.spec_cap : 0;
     if ((err = copy_on(h, h->d_ns + e, &S, sizeof(S), cudaMemcpyHostToDevice)) ||
+        (err = copy_on(h, &dt->spec_cap, &task_cap, sizeof(int32_t), cudaMemcpyHostToDevice)) ||
         (err = copy_on(h, &dt->done, &S.done, sizeof(int32_t), cudaMemcpyHostToDevice)) ||
         (err = copy_on(h, &dt->n_steps, &S.n_steps, sizeof(int32_t), cudaMemcpyHostToDevice)) ||
         (err = copy_on(h, &dt->spec, &S.spec, sizeof(int32_t), cudaMemcpyHostToDevice)))

@@ -108,6 +108,7 @@ extern "C" int ns_walk_batch_noalloc(ns_handle* h, int event, const double* live
   T.done = 0;
   T.event = event;
   T.spec = E.cfg.spec_depth > 0 ? E.cfg.spec_depth : default_spec(h->precision);
+  T.spec_cap = E.cfg.spec_depth > 0 ? 0 : kSpecMax;
   watchdog_fields(h, T);
   cudaStream_t s = stream ? (cudaStream_t)stream : h->stream;
   // the flow kernels' timeout flag and the walk watchdog's bit start clear, as in ns_walk_batch
