@@ -123,7 +123,7 @@ static int prepare_event(ns_handle* h, int e, const ns_config& c, const ns_event
   const int nbas = c.waveform == NS_WAVEFORM_PHENOMD_FORM ? kBasisPD : kBasis;
   std::vector<double> basis((size_t)nb * nbas);
   std::vector<float2> basis_ff((size_t)nb * nbas);
-  std::vector<double> gw64((size_t)nd * nb);
+  std::vector<double> gw64((size_t)nd * nb), a76(nb);
   std::vector<float> gw32((size_t)nd * nb);
   std::vector<double2> z64((size_t)nd * nb);
   std::vector<float2> z32((size_t)nd * nb);
@@ -132,6 +132,7 @@ static int prepare_event(ns_handle* h, int e, const ns_config& c, const ns_event
   for (int k = 0; k < nb; ++k) {
     double f = in.f_min + in.df * (double)k;
     double c3 = std::cbrt(f), lf = std::log(f);
+    a76[k] = std::pow(f, -7.0 / 6.0);
     double* g = &basis[(size_t)k * nbas];
     g[0] = 1.0 / (f * c3 * c3);   // f^-5/3
     g[1] = 1.0 / f;               // f^-1
@@ -158,9 +159,8 @@ static int prepare_event(ns_handle* h, int e, const ns_config& c, const ns_event
     const ns_detector& det = in.det[d];
     double run = 0.0, runc = 0.0;
     for (int k = 0; k < nb; ++k) {
-      double f = in.f_min + in.df * (double)k;
       double w = 4.0 * in.df / det.psd[k];
-      double a = std::pow(f, -7.0 / 6.0);
+      double a = a76[k];
       double zr = w * det.d_re[k] * a, zi = -w * det.d_im[k] * a;   // 4 df conj(d) f^-7/6 / S
       z64[(size_t)d * nb + k] = make_double2(zr, zi);
       z32[(size_t)d * nb + k] = make_float2((float)zr, (float)zi);
@@ -193,6 +193,7 @@ static int prepare_event(ns_handle* h, int e, const ns_config& c, const ns_event
       (err = cudaMalloc(&E.d_z32, z32.size() * sizeof(float2))) != cudaSuccess ||
       (err = cudaMalloc(&E.d_hh_prefix, pref.size() * sizeof(double))) != cudaSuccess ||
       (err = cudaMalloc(&E.d_gw64, gw64.size() * sizeof(double))) != cudaSuccess ||
+      (err = cudaMalloc(&E.d_a76, a76.size() * sizeof(double))) != cudaSuccess ||
       (err = cudaMalloc(&E.d_gw32, gw32.size() * sizeof(float))) != cudaSuccess ||
       (err = cudaMalloc(&E.d_hhp32, pref32.size() * sizeof(float))) != cudaSuccess)
     return set_error(nullptr, NS_ENOMEM, "event %d: device allocation failed: %s", e, cudaGetErrorString(err));
@@ -201,6 +202,7 @@ static int prepare_event(ns_handle* h, int e, const ns_config& c, const ns_event
       (err = copy_on(h, E.d_z64, z64.data(), z64.size() * sizeof(double2), cudaMemcpyHostToDevice)) != cudaSuccess ||
       (err = copy_on(h, E.d_z32, z32.data(), z32.size() * sizeof(float2), cudaMemcpyHostToDevice)) != cudaSuccess ||
       (err = copy_on(h, E.d_hh_prefix, pref.data(), pref.size() * sizeof(double), cudaMemcpyHostToDevice)) != cudaSuccess ||
+      (err = copy_on(h, E.d_a76, a76.data(), a76.size() * sizeof(double), cudaMemcpyHostToDevice)) != cudaSuccess ||
       (err = copy_on(h, E.d_gw64, gw64.data(), gw64.size() * sizeof(double), cudaMemcpyHostToDevice)) != cudaSuccess ||
       (err = copy_on(h, E.d_gw32, gw32.data(), gw32.size() * sizeof(float), cudaMemcpyHostToDevice)) != cudaSuccess ||
       (err = copy_on(h, E.d_hhp32, pref32.data(), pref32.size() * sizeof(float), cudaMemcpyHostToDevice)) != cudaSuccess)
@@ -282,6 +284,7 @@ static int prepare_event(ns_handle* h, int e, const ns_config& c, const ns_event
   D.dd_f[0] = (float)dd;
   D.dd_f[1] = (float)(dd - (double)D.dd_f[0]);
   D.gw64 = E.d_gw64;
+  D.a76 = E.d_a76;
   D.gw32 = E.d_gw32;
   D.gw32_unscale = 1.0 / gscale;
   D.hh_unscale_f = (float)std::ldexp(D.gw32_unscale, -2 * kKpScaleExp);
@@ -299,6 +302,8 @@ void free_event(EventHost& E) {
   cudaFree(E.d_hhp32);
   E.d_hhp32 = nullptr;
   cudaFree(E.d_gw64);
+  cudaFree(E.d_a76);
+  E.d_a76 = nullptr;
   cudaFree(E.d_gw32);
   E.d_gw64 = nullptr;
   E.d_gw32 = nullptr;

@@ -64,6 +64,7 @@ struct EventHost {
   float2* d_z32 = nullptr;
   double* d_hh_prefix = nullptr;
   double* d_gw64 = nullptr;
+  double* d_a76 = nullptr;
   float* d_gw32 = nullptr;
   float* d_hhp32 = nullptr;
   int32_t* d_rb_edges = nullptr;   // relative binning (relbin.cu)

@@ -79,6 +79,7 @@ struct EventDev {
   const double2* z64;                  // [n_det][n_bins]
   const float2* z32;                   // [n_det][n_bins]
   const double* hh_prefix;             // [n_det][n_bins] inclusive prefix sums of 4 df f^-7/3 / S
+  const double* a76;                   // [n_bins] f^-7/6
   const double* gw64;                  // [n_det][n_bins] 4 df f^-7/3 / S (per-bin template power)
   const float* gw32;                   // [n_det][n_bins] FP32 copy scaled by 1/gw32_unscale (a power
                                        //   of two: the weights reach ~1e43, beyond FP32's range)

@@ -14,6 +14,7 @@
 
 #include "flow.cuh"
 #include "gwns_internal.h"
+#include "setup_split.cuh"
 
 namespace gwns {
 
@@ -549,77 +550,62 @@ __device__ inline void setup_from_theta(const EventDev& ev, const double* th, Wa
 }
 
 // ---------------------------------------------------------------- likelihood batch
-template <int PREC, int NDET, int WF>
-__global__ void __launch_bounds__(kThreads) likelihood_kernel(const EventDev* __restrict__ evp,
-                                                               const double* __restrict__ theta, int n,
-                                                               double* __restrict__ lnl, int32_t* status) {
-  __shared__ WalkerParams P;
-  __shared__ double red[kWarps][NVals<NDET, WF>::value];
-  __shared__ double vals[kMaxVals];
-  __shared__ int ok;
+// ln L of n proposals, in [n][11] physical vectors or (UNIT) [n][D] unit-cube points: one CTA takes a
+// tile of `tile` of them.  The four warps form the tile's constants together (setup_tile: a
+// proposal a lane), then the likelihoods run in the walks' summation order.  With one proposal a
+// CTA, one thread formed its constants while the other 127 waited (barrier stalls 33 of every 48
+// warp cycles, the FP64 pipe busy with one lane in 32).  Non-finite vectors: NaN and status; UNIT
+// (the initial live points): non-finite results become -inf, so that they die first.
+constexpr int kLikTile = 16;
+
+template <int PREC, int NDET, int WF, bool UNIT>
+__global__ void __launch_bounds__(kThreads, 4) likelihood_kernel(const EventDev* __restrict__ evp,
+                                                                 const double* __restrict__ in, int n, int tile,
+                                                                 double* __restrict__ lnl, int32_t* status) {
+  constexpr int NV = NVals<NDET, WF>::value;
+  __shared__ WalkerParams P[kLikTile];
+  __shared__ TilePart<PREC, WF> parts[kLikTile];
+  __shared__ double ct[kWarps][kWarps][NV];
+  __shared__ double tot[kLikTile][NV];
+  __shared__ double rbl[kLikTile];
+  __shared__ int ok[kLikTile];
   const EventDev& ev = *evp;
-  const int w = blockIdx.x;
-  if (threadIdx.x == 0) {
-    double th[kParams];
-    for (int i = 0; i < kParams; ++i) th[i] = theta[(size_t)w * kParams + i];
-    ok = theta_ok(th);
-    if (ok) setup_from_theta<PREC, WF>(ev, th, P);
-    else P.k_end = 0;
+  const int base = blockIdx.x * tile, m = min(tile, n - base);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const double* v = in + (size_t)base * (UNIT ? ev.n_dim : kParams);
+  if ((int)threadIdx.x < m) ok[threadIdx.x] = UNIT ? 1 : (theta_ok(v + (size_t)threadIdx.x * kParams) ? 1 : 0);
+  __syncthreads();
+  setup_tile<PREC, WF, UNIT>(ev, v, m, ok, parts, P);
+  bool rb = false;
+  if constexpr (PREC == 2) rb = ev.rb_nb > 0;
+  if (rb) {
+    if constexpr (PREC == 2) {   // relative binning: a warp per proposal
+      for (int i = warp; i < m; i += kWarps) {
+        const double l = ok[i] ? rb_lnl_warp<NDET, WF>(ev, P[i], lane) : 0.0;
+        if (lane == 0) rbl[i] = l;
+      }
+    }
+  } else if (WF == 0 && m >= kWarps) {
+    // hundreds of bins: a warp per proposal, its four chunks in turn, no barrier between proposals
+    for (int i = warp; i < m; i += kWarps) {
+      warp_chunks<PREC, NDET, WF>(ev, P[i], lane, ct[warp]);
+      if (lane < NV) tot[i][lane] = chunks_sum<NV>(ct[warp], lane);
+      __syncwarp();
+    }
+  } else {
+    for (int i = 0; i < m; ++i) cta_sums<PREC, NDET, WF>(ev, P[i], ct[0], tot[i]);
   }
   __syncthreads();
-  if constexpr (PREC == 2) {
-    if (ev.rb_nb > 0) {   // relative binning: warp 0 evaluates the proposal
-      if (threadIdx.x < 32) {
-        const double v = ok ? rb_lnl_warp<NDET, WF>(ev, P, threadIdx.x) : 0.0;
-        if (threadIdx.x == 0) {
-          if (ok) {
-            lnl[w] = v;
-          } else {
-            lnl[w] = __longlong_as_double(0x7ff8000000000000ll);
-            atomicOr(status, 1);
-          }
-        }
-      }
-      return;
-    }
-  }
-  cta_sums<PREC, NDET, WF>(ev, P, red, vals);
-  if (threadIdx.x == 0) {
-    if (ok) {
-      lnl[w] = lnl_from_vals<PREC, NDET, WF>(ev, P, vals);
-    } else {
-      lnl[w] = __longlong_as_double(0x7ff8000000000000ll);
+  if ((int)threadIdx.x < m) {
+    const int i = threadIdx.x;
+    double l = rb ? rbl[i] : lnl_from_vals<PREC, NDET, WF>(ev, P[i], tot[i]);
+    if (UNIT) {
+      l = isfinite(l) ? l : -INFINITY;
+    } else if (!ok[i]) {
+      l = __longlong_as_double(0x7ff8000000000000ll);
       atomicOr(status, 1);
     }
-  }
-}
-
-// ln L of unit-cube points u [n][D] (prior transform, then the likelihood).  Used for the
-// initial live points; non-finite results are stored as -inf so that they die first.
-template <int PREC, int NDET, int WF>
-__global__ void __launch_bounds__(kThreads) unit_likelihood_kernel(const EventDev* __restrict__ evp,
-                                                                    const double* __restrict__ u, int n,
-                                                                    double* __restrict__ lnl) {
-  __shared__ WalkerParams P;
-  __shared__ double red[kWarps][NVals<NDET, WF>::value];
-  __shared__ double vals[kMaxVals];
-  const EventDev& ev = *evp;
-  const int w = blockIdx.x;
-  if (threadIdx.x == 0) setup_from_unit<PREC, WF>(ev, u + (size_t)w * ev.n_dim, P);
-  __syncthreads();
-  if constexpr (PREC == 2) {
-    if (ev.rb_nb > 0) {
-      if (threadIdx.x < 32) {
-        const double v = rb_lnl_warp<NDET, WF>(ev, P, threadIdx.x);
-        if (threadIdx.x == 0) lnl[w] = isfinite(v) ? v : -INFINITY;
-      }
-      return;
-    }
-  }
-  cta_sums<PREC, NDET, WF>(ev, P, red, vals);
-  if (threadIdx.x == 0) {
-    double v = lnl_from_vals<PREC, NDET, WF>(ev, P, vals);
-    lnl[w] = isfinite(v) ? v : -INFINITY;
+    lnl[base + i] = l;
   }
 }
 
@@ -635,35 +621,44 @@ __global__ void unit_to_theta_kernel(const EventDev* __restrict__ evp, const dou
 }
 
 // ---------------------------------------------------------------- waveform (FP64)
+// Detector strains of theta blockIdx.y in the bins [span blockIdx.x, span (blockIdx.x + 1)).  The
+// CTA forms the constants on its four warps, once for the whole span (a CTA per 256 bins formed
+// them on one thread, 64 times a vector at 16,225 bins).
 template <int NDET, int WF>
-__global__ void __launch_bounds__(256) waveform_kernel(const EventDev* __restrict__ evp,
-                                                       const double* __restrict__ theta, int n_bins,
-                                                       double* __restrict__ h_re, double* __restrict__ h_im,
-                                                       int no_cutoff) {
+__global__ void __launch_bounds__(kThreads) waveform_kernel(const EventDev* __restrict__ evp,
+                                                            const double* __restrict__ theta, int n_bins, int span,
+                                                            double* __restrict__ h_re, double* __restrict__ h_im,
+                                                            int no_cutoff) {
   __shared__ WalkerParams P;
+  __shared__ TilePart<0, WF> part;
+  __shared__ int ok;
   const EventDev& ev = *evp;
   const int w = blockIdx.y;
-  if (threadIdx.x == 0) {
-    double th[kParams];
-    for (int i = 0; i < kParams; ++i) th[i] = theta[(size_t)w * kParams + i];
-    setup_from_theta<0, WF>(ev, th, P);
-    if (no_cutoff) P.k_end = n_bins;
-  }
+  if (threadIdx.x == 0) ok = 1;
   __syncthreads();
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= n_bins) return;
-  const double f = ev.f_min + ev.df * (double)k;
-  double phi = 0.0, amp = 0.0;
-  if (k < P.k_end) {
+  setup_tile<0, WF, false>(ev, theta + (size_t)w * kParams, 1, &ok, &part, &P);
+  const int k_end = no_cutoff ? n_bins : P.k_end;
+  const int last = min((int)(blockIdx.x + 1) * span, n_bins);
+  for (int k = blockIdx.x * span + threadIdx.x; k < last; k += kThreads) {
+    const size_t o0 = (size_t)w * NDET * n_bins + k;
+    if (k >= k_end) {
+#pragma unroll
+      for (int det = 0; det < NDET; ++det) h_re[o0 + (size_t)det * n_bins] = h_im[o0 + (size_t)det * n_bins] = 0.0;
+      continue;
+    }
+    const double f = ev.f_min + ev.df * (double)k;
     const double* g = ev.basis64 + (size_t)k * ev.n_basis;
+    double phi, amp;
     if (WF == 0) {
       phi = P.phase0;
+#pragma unroll
       for (int j = 0; j < kBasis; ++j) phi = fma(P.C[j], g[j], phi);
       amp = 1.0;
     } else {
       const PhenomExtra& e = P.pd;
       if (k < e.k1) {
         phi = P.phase0;
+#pragma unroll
         for (int j = 0; j < kBasis; ++j) phi = fma(P.C[j], g[j], phi);
         phi = fma(e.Cx[0], g[8], fma(e.Cx[1], g[9], fma(e.Cx[2], g[10], phi)));
       } else if (k < e.k2) {
@@ -674,23 +669,15 @@ __global__ void __launch_bounds__(256) waveform_kernel(const EventDev* __restric
       }
       amp = pd_amp_f64(e, k, f, g[4]);
     }
-  }
-  const double a7 = pow(f, -7.0 / 6.0) * amp;
+    const double a7 = ev.a76[k] * amp;
 #pragma unroll
-  for (int det = 0; det < NDET; ++det) {
-    double re = 0.0, im = 0.0;
-    if (k < P.k_end) {
-      double ph = fma(P.tau[det], f, phi);
-      double r = ph - rint(ph);
+    for (int det = 0; det < NDET; ++det) {
       double s, c;
-      sincospi(2.0 * r, &s, &c);
-      // a f^-7/6 K P exp(-2 pi i r)
-      re = a7 * (P.kp_re[det] * c + P.kp_im[det] * s);
-      im = a7 * (P.kp_im[det] * c - P.kp_re[det] * s);
+      sincos_phase_f64(fma(P.tau[det], f, phi), &s, &c);
+      // a f^-7/6 K P exp(-2 pi i ph)
+      h_re[o0 + (size_t)det * n_bins] = a7 * (P.kp_re[det] * c + P.kp_im[det] * s);
+      h_im[o0 + (size_t)det * n_bins] = a7 * (P.kp_im[det] * c - P.kp_re[det] * s);
     }
-    size_t o = ((size_t)w * NDET + det) * n_bins + k;
-    h_re[o] = re;
-    h_im[o] = im;
   }
 }
 
@@ -1926,10 +1913,20 @@ __global__ void __launch_bounds__(kThreads, 4) hrss_kernel_ff(const EventDev* __
 #define GWNS_DISPATCH_W(K, P)                                                     \
   if (waveform == 0) { GWNS_DISPATCH_N(K, P, 0) } else { GWNS_DISPATCH_N(K, P, 1) }
 
+// Proposals of a CTA: as many as keep every SM at two CTAs (a setup costs its warps the same FP64
+// time for one proposal or for a full tile), up to 16 for TaylorF2; up to 4 for the IMRPhenomD
+// form, whose evaluations take ~100 times a setup and balance better in small pieces.
+inline int lik_tile(int n, int waveform) {
+  const int t = (n + 303) / 304, most = waveform == 0 ? kLikTile : 4;
+  return t < 1 ? 1 : (t > most ? most : t);
+}
+
 template <int P>
 cudaError_t launch_likelihood_p(int waveform, int n_det, const EventDev* d_ev, const double* d_theta, int n,
                                 double* d_lnl, int32_t* d_status, cudaStream_t s) {
-#define GWNS_LIK(P_, N, W) likelihood_kernel<P_, N, W><<<n, kThreads, 0, s>>>(d_ev, d_theta, n, d_lnl, d_status)
+  const int tile = lik_tile(n, waveform), grid = (n + tile - 1) / tile;
+#define GWNS_LIK(P_, N, W) \
+  likelihood_kernel<P_, N, W, false><<<grid, kThreads, 0, s>>>(d_ev, d_theta, n, tile, d_lnl, d_status)
   GWNS_DISPATCH_W(GWNS_LIK, P)
 #undef GWNS_LIK
   return cudaGetLastError();
@@ -1938,14 +1935,15 @@ cudaError_t launch_likelihood_p(int waveform, int n_det, const EventDev* d_ev, c
 template <int P>
 cudaError_t launch_unit_likelihood_p(int waveform, int n_det, const EventDev* d_ev, const double* d_u, int n,
                                      double* d_lnl, cudaStream_t s) {
-#define GWNS_UL(P_, N, W) unit_likelihood_kernel<P_, N, W><<<n, kThreads, 0, s>>>(d_ev, d_u, n, d_lnl)
+  const int tile = lik_tile(n, waveform), grid = (n + tile - 1) / tile;
+#define GWNS_UL(P_, N, W) \
+  likelihood_kernel<P_, N, W, true><<<grid, kThreads, 0, s>>>(d_ev, d_u, n, tile, d_lnl, nullptr)
   GWNS_DISPATCH_W(GWNS_UL, P)
 #undef GWNS_UL
   return cudaGetLastError();
 }
 
-// Mode 2 runs the float-float walk; modes 0 and 1 the FP64-recheck walk.  A TaylorF2 launch
-// whose tasks use neither flow proposals nor the relative-binning likelihood (extras false)
+// Mode 2 runs the float-float walk; modes 0 and 1 the FP64-recheck walk.  A launch whose tasks use neither flow proposals nor the relative-binning likelihood (extras false)
 // runs the float-float walk compiled without those paths (a smaller kernel: its round is
 // short and instruction fetch is among its first stalls).  Both properties of an event are
 // fixed before its first ns_step (ns_relbin_set is refused after it), so the sampler's
@@ -1954,7 +1952,7 @@ template <int P, int N, int W>
 void launch_walk_one(int n_blocks, cudaStream_t s, const EventDev* d_evs, WalkTask* d_tasks,
                      const int32_t* d_blk_task, const int32_t* d_blk_local, bool extras) {
   if constexpr (P == 2) {
-    if (W == 0 && !extras)
+    if (!extras)
       walk_kernel_ff<N, W, false><<<n_blocks, kThreads, 0, s>>>(d_evs, d_tasks, d_blk_task, d_blk_local);
     else
       walk_kernel_ff<N, W, true><<<n_blocks, kThreads, 0, s>>>(d_evs, d_tasks, d_blk_task, d_blk_local);
