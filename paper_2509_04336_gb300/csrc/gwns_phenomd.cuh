@@ -176,13 +176,15 @@ __device__ __forceinline__ double pd_amp_f64(const PhenomExtra& e, int k, double
   return e.g1gd / (d * d + e.gd * e.gd) * exp(-e.g2_gd * d);
 }
 
+// AM: the amplitude region (0 inspiral, 1 intermediate, 2 merger-ringdown; -1: by k)
+template <int AM = -1>
 __device__ __forceinline__ float pd_amp_f32(const PhenomExtra& e, int k, float f, float f13) {
-  if (k < e.ka) {
+  if (AM == 0 || (AM < 0 && k < e.ka)) {
     float v = e.c13f * f13;
     return 1.0f + e.A2f * v * v + e.A3f * v * v * v;
   }
   float x = e.Mf * f;
-  if (k < e.kp) {
+  if (AM == 1 || (AM < 0 && k < e.kp)) {
     float s = (x - e.xaf) * e.inv_spanf;
     return e.hy0f + s * (e.hd0f + s * (e.hc2f + s * e.hc3f));
   }
@@ -294,50 +296,75 @@ __device__ __forceinline__ void ff_term(float& sh, float& sl, float ch, float cl
   sl += err + e;
 }
 
-template <int NDET>
-__device__ __forceinline__ void pd_accumulate_ff(const EventDev& ev, const WalkerParams& p, const PhenomExtra& e, int k,
-                                                 AccPD32& acc) {
-  const float2* g = ev.basis_ff + k;
+// The bins k, k + stride, ... below `end` of one proposal, whose phase region PH (0 inspiral,
+// 1 intermediate, 2 merger-ringdown) and amplitude region AM (the same) are known; -1: found bin by
+// bin.  On return k is the thread's first bin at or above `end`.
+template <int NDET, int PH, int AM>
+__device__ __forceinline__ void pd_segment_ff(const EventDev& ev, const WalkerParams& p, const PhenomExtra& e, int& k,
+                                              int end, int stride, AccPD32& acc) {
   const size_t gs = (size_t)ev.n_bins;
-  const float ff = g[13 * gs].x;   // f (exact on the grids used: f_min + k df in FP32)
-  float sh, sl, extra = 0.f;
-  if (k < e.k1) {
-    sh = p.ph0h; sl = p.ph0l;
+#pragma unroll 1
+  for (; k < end; k += stride) {
+    const float2* g = ev.basis_ff + k;
+    const float ff = g[13 * gs].x;   // f (exact on the grids used: f_min + k df in FP32)
+    float sh, sl, extra = 0.f;
+    if (PH == 0 || (PH < 0 && k < e.k1)) {
+      sh = p.ph0h; sl = p.ph0l;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) ff_term(sh, sl, p.Ch[j], p.Cl[j], g[j * gs]);
-    ff_term(sh, sl, e.Cxh[0], e.Cxl[0], g[8 * gs]);
-    ff_term(sh, sl, e.Cxh[1], e.Cxl[1], g[9 * gs]);
-    ff_term(sh, sl, e.Cxh[2], e.Cxl[2], g[10 * gs]);
-  } else if (k < e.k2) {
-    sh = e.ph0_int_h; sl = e.ph0_int_l;
-    ff_term(sh, sl, e.Cxh[3], e.Cxl[3], g[6 * gs]);
-    ff_term(sh, sl, e.Cxh[4], e.Cxl[4], g[11 * gs]);
-    ff_term(sh, sl, e.Cxh[5], e.Cxl[5], g[13 * gs]);
-  } else {
-    sh = e.ph0_mr_h; sl = e.ph0_mr_l;
-    ff_term(sh, sl, e.Cxh[6], e.Cxl[6], g[1 * gs]);
-    ff_term(sh, sl, e.Cxh[7], e.Cxl[7], g[12 * gs]);
-    ff_term(sh, sl, e.Cxh[8], e.Cxl[8], g[13 * gs]);
-    extra = e.at_scalef * atanf((e.Mf * ff - e.at_cf) * e.at_invf);
+      for (int j = 0; j < 8; ++j) ff_term(sh, sl, p.Ch[j], p.Cl[j], g[j * gs]);
+      ff_term(sh, sl, e.Cxh[0], e.Cxl[0], g[8 * gs]);
+      ff_term(sh, sl, e.Cxh[1], e.Cxl[1], g[9 * gs]);
+      ff_term(sh, sl, e.Cxh[2], e.Cxl[2], g[10 * gs]);
+    } else if (PH == 1 || (PH < 0 && k < e.k2)) {
+      sh = e.ph0_int_h; sl = e.ph0_int_l;
+      ff_term(sh, sl, e.Cxh[3], e.Cxl[3], g[6 * gs]);
+      ff_term(sh, sl, e.Cxh[4], e.Cxl[4], g[11 * gs]);
+      ff_term(sh, sl, e.Cxh[5], e.Cxl[5], g[13 * gs]);
+    } else {
+      sh = e.ph0_mr_h; sl = e.ph0_mr_l;
+      ff_term(sh, sl, e.Cxh[6], e.Cxl[6], g[1 * gs]);
+      ff_term(sh, sl, e.Cxh[7], e.Cxl[7], g[12 * gs]);
+      ff_term(sh, sl, e.Cxh[8], e.Cxl[8], g[13 * gs]);
+      extra = e.at_scalef * atanf((e.Mf * ff - e.at_cf) * e.at_invf);
+    }
+    const float r0 = (sh - rintf(sh)) + sl + extra;
+    const float amp = pd_amp_f32<AM>(e, k, ff, (AM <= 0) ? g[4 * gs].x : 0.0f);
+    const float amp2 = amp * amp;
+    const float kf = (float)k;
+#pragma unroll
+    for (int det = 0; det < NDET; ++det) {
+      float kb = kf * p.sbh[det];
+      float x = kb - rintf(kb);
+      float ph = (r0 + p.sa[det]) + x + kf * p.sbl[det];
+      ph = ph - rintf(ph);
+      float s, c;
+      sincos_turn_sfu(ph, &s, &c);
+      float2 z = ev.z32[(size_t)det * ev.n_bins + k];
+      kahan_add(acc.re[det], acc.cre[det], amp * fmaf(z.x, c, z.y * s));
+      kahan_add(acc.im[det], acc.cim[det], amp * fmaf(z.y, c, -z.x * s));
+      // template power: positive terms, no cancellation -- a plain FP32 sum per lane (the lanes'
+      // sums are combined with error-free additions)
+      acc.hh[det] = fmaf(amp2, ev.gw32[(size_t)det * ev.n_bins + k], acc.hh[det]);
+    }
   }
-  const float r0 = (sh - rintf(sh)) + sl + extra;
-  const float amp = pd_amp_f32(e, k, ff, g[4 * gs].x);
-  const float amp2 = amp * amp;
-  const float kf = (float)k;
-#pragma unroll
-  for (int det = 0; det < NDET; ++det) {
-    float kb = kf * p.sbh[det];
-    float x = kb - rintf(kb);
-    float ph = (r0 + p.sa[det]) + x + kf * p.sbl[det];
-    ph = ph - rintf(ph);
-    float s, c;
-    sincos_turn_sfu(ph, &s, &c);
-    float2 z = ev.z32[(size_t)det * ev.n_bins + k];
-    kahan_add(acc.re[det], acc.cre[det], amp * fmaf(z.x, c, z.y * s));
-    kahan_add(acc.im[det], acc.cim[det], amp * fmaf(z.y, c, -z.x * s));
-    // template power: positive terms, no cancellation -- a plain FP32 sum per lane (the lanes'
-    // sums are combined with error-free additions)
-    acc.hh[det] = fmaf(amp2, ev.gw32[(size_t)det * ev.n_bins + k], acc.hh[det]);
+}
+
+// The bins k, k + stride, ... < k_end of one proposal, region by region: a loop per region keeps
+// only that region's constants in registers (the loop with a branch a bin kept every region's,
+// spilled, and read the rest from shared memory at each bin).  A lane's bins are summed in
+// ascending order either way.  4,001 likelihoods of 16,225 bins 579 -> 470 us; the walk of 1000
+// walkers x 240 steps 20.8 -> 20.2 ms.
+template <int NDET>
+__device__ __forceinline__ void pd_sums_ff(const EventDev& ev, const WalkerParams& p, const PhenomExtra& e, int k,
+                                           int k_end, int stride, AccPD32& acc) {
+  if (e.ka <= e.k1 && e.k1 <= e.k2 && e.k2 <= e.kp) {   // the order of every physical proposal
+    pd_segment_ff<NDET, 0, 0>(ev, p, e, k, min(e.ka, k_end), stride, acc);
+    pd_segment_ff<NDET, 0, 1>(ev, p, e, k, min(e.k1, k_end), stride, acc);
+    pd_segment_ff<NDET, 1, 1>(ev, p, e, k, min(e.k2, k_end), stride, acc);
+    pd_segment_ff<NDET, 2, 1>(ev, p, e, k, min(e.kp, k_end), stride, acc);
+    pd_segment_ff<NDET, 2, 2>(ev, p, e, k, k_end, stride, acc);
+  } else {
+    pd_segment_ff<NDET, -1, -1>(ev, p, e, k, k_end, stride, acc);
   }
 }
 

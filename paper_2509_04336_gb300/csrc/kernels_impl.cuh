@@ -96,7 +96,7 @@ __device__ inline void partials(const EventDev& ev, const WalkerParams& P, int s
       if (PREC == 1) {
         for (int k = start; k < P.k_end; k += stride) pd_accumulate_mixed<NDET>(ev, P, P.pd, k, acc);
       } else {
-        for (int k = start; k < P.k_end; k += stride) pd_accumulate_ff<NDET>(ev, P, P.pd, k, acc);
+        pd_sums_ff<NDET>(ev, P, P.pd, start, P.k_end, stride, acc);
       }
 #pragma unroll
       for (int d = 0; d < NDET; ++d) {
@@ -488,7 +488,7 @@ __device__ double rb_lnl_warp(const EventDev& ev, const WalkerParams& P, int lan
   } else {
     AccPD32 acc;
     acc.zero();
-    for (int k = kx + lane; k < k_end; k += 32) pd_accumulate_ff<NDET>(ev, P, P.pd, k, acc);
+    pd_sums_ff<NDET>(ev, P, P.pd, kx + lane, k_end, 32, acc);
     float sdh = 0.f, shh = 0.f;
 #pragma unroll
     for (int det = 0; det < NDET; ++det) {
