@@ -706,8 +706,8 @@ __device__ __forceinline__ int round_depth(const WalkTask& T, int n_acc, int n_l
 //     current position; the candidates that may lie in the cube are compacted into one warp,
 //     which redoes their draws and proposals exactly in FP64 and compacts the in-bounds ones,
 //     in step order, into at most m = task.spec slots;
-//  2. that warp computes the per-proposal constants (the FP64-heavy part) on full lanes, and
-//     the CTA evaluates the slots' likelihoods, one warp per proposal (the whole CTA per
+//  2. the four warps form the per-proposal constants together (independent chains on different
+//     warps, a proposal a lane), and the CTA evaluates the slots' likelihoods, one warp per proposal (the whole CTA per
 //     proposal when there are fewer than kWarps of them);
 //  3. thread 0 replays the steps in order: out-of-bounds steps reject without a likelihood
 //     call, the first in-bounds proposal with ln L > ln L* is taken and ends the round.
@@ -727,6 +727,7 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel(const EventDev* __res
                                                          const int32_t* __restrict__ blk_local) {
   constexpr int NV = NVals<NDET, WF>::value;
   __shared__ WalkerParams P[kSpecMax];
+  __shared__ SetupPart parts[kSpecMax];
   __shared__ double prop[kSpecMax][kMaxDim];
   __shared__ int cstep[kSpecMax];
   __shared__ int mstep[32];
@@ -914,13 +915,17 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel(const EventDev* __res
       else if (total > 32) end = __shfl_sync(0xffffffffu, st, 31);
       else end = t + W - 1;
       if (lane == 0) { s_nin = nin_w; s_end = end; }
-      __syncwarp();
-      if (lane < nin_w) setup_from_unit<PREC, WF>(ev, prop[lane], P[lane]);
     }
     __syncthreads();
     const int nin = s_nin;
-    // 2. likelihoods: the sums of proposal i into tot_p[i] (chunk totals in ct), then one lane
+    // 2. proposal constants on all four warps (setup_split.cuh), then the likelihoods: the sums of proposal i into tot_p[i] (chunk totals in ct), then one lane
     //    per proposal assembles ln L (the FP64 part runs once per proposal, on one warp)
+    if (nin > 0) {
+      if (lane < nin) f64_split_first<PREC != 0, true>(warp, ev, prop[lane], parts[lane], P[lane]);
+      __syncthreads();
+      if (lane < nin) f64_split_second<PREC != 0, WF>(warp, ev, parts[lane], P[lane]);
+      __syncthreads();
+    }
     if (nin >= kWarps) {
       // one warp per proposal, its four chunks in turn
       for (int i = warp; i < nin; i += kWarps) {
