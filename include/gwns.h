@@ -115,9 +115,9 @@ typedef struct ns_config {
     int32_t max_iter;     /* hard cap on batches (0: 1000000)                       */
     int32_t n_steps0;     /* first walk length (0: ceil(naccept / 0.25))            */
     uint64_t seed;        /* Philox key word 0; key word 1 is the event index      */
-    int32_t spec_depth;   /* walk steps evaluated per round (1..32); 0: chosen per batch, and
-                             within it per walker, from the acceptance rate.  Any value gives
-                             the same chain.                                             */
+    int32_t spec_depth;   /* walk steps evaluated per round (1..32); 0: chosen per batch (in a
+                             stand-alone walk per walker) from the acceptance rate.  Any
+                             value gives the same chain.                                 */
     int32_t proposal;     /* NS_PROPOSAL_DE, or NS_PROPOSAL_DE_FLOW: DE steps mixed with
                              independence proposals from a normalising flow trained on the
                              live points (see "Flow proposal" below)                  */

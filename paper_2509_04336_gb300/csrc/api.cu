@@ -541,7 +541,7 @@ extern "C" int ns_walk_batch(ns_handle* h, int event, const double* live_u, int 
         (e = cudaMemcpyAsync(d_l0, lnl0, sizeof(double) * n, cudaMemcpyHostToDevice, s)))
       return cuda_fail(h, e, "H2D walk inputs");
     if ((e = launch_walk_prepare(T, d_task, d_be, d_bl, d_survf, clear, ns_, s)) != cudaSuccess ||
-        (e = launch_walk(h->precision, h->waveform, E.n_det, h->d_events, d_task, d_be, d_bl, n, s, walk_extras(h, event))) != cudaSuccess)
+        (e = launch_walk(h->precision, h->waveform, E.n_det, h->d_events, d_task, d_be, d_bl, n, s, walk_extras(h, event), true)) != cudaSuccess)
       return cuda_fail(h, e, "walk launch");
     if ((e = cudaMemcpyAsync(u_out, d_uo, sizeof(double) * nu, cudaMemcpyDeviceToHost, s)) ||
         (e = cudaMemcpyAsync(lnl_out, d_lo, sizeof(double) * n, cudaMemcpyDeviceToHost, s)) ||
@@ -556,7 +556,7 @@ extern "C" int ns_walk_batch(ns_handle* h, int event, const double* live_u, int 
   T.surv = live_u; T.u0 = u0; T.lnl0 = lnl0; T.u_out = u_out; T.lnl_out = lnl_out; T.n_acc = n_accept; T.n_like = n_like;
   if ((e = launch_walk_prepare(T, d_task, d_be, d_bl, d_survf, clear, ns_, s)) != cudaSuccess)
     return cuda_fail(h, e, "walk task launch");
-  e = launch_walk(h->precision, h->waveform, E.n_det, h->d_events, d_task, d_be, d_bl, n, s, walk_extras(h, event));
+  e = launch_walk(h->precision, h->waveform, E.n_det, h->d_events, d_task, d_be, d_bl, n, s, walk_extras(h, event), true);
   return e == cudaSuccess ? NS_OK : cuda_fail(h, e, "walk launch");
 }
 

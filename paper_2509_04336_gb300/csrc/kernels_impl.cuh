@@ -681,21 +681,37 @@ __global__ void __launch_bounds__(kThreads) waveform_kernel(const EventDev* __re
   }
 }
 
-// Proposals of a walker's next round, from its own n_acc acceptances in n_like calls so far: the
-// rule of the batch retune, about 1.4 / p in-bounds proposals at p acceptances a call (the first
-// acceptance then falls on average in the first two thirds of the round), with the task's depth
-// as the first estimate, worth 1.4 acceptances.  Walkers of one batch differ in p by several
-// times, and a stand-alone walk has no batch before it: a fixed depth of 16 dropped 9 of 10
-// evaluations at p = 0.6.  A depth fixed by the user (spec_cap 0) stays.  Any depth gives the
-// same chain.  PAD4: rounds of a warp per proposal, padded to a multiple of four.
-template <bool PAD4>
-__device__ __forceinline__ int round_depth(const WalkTask& T, int n_acc, int n_like) {
-  int m = T.spec < 1 ? 1 : (T.spec > kSpecMax ? kSpecMax : T.spec);
+// A walker's next round, from its own n_acc acceptances in n_like calls so far: `depth` proposals,
+// looking ahead over rejections or (`chain`) over acceptances.
+//   A DE move's difference does not depend on the position, so the proposals of later steps follow
+// from any guess at the earlier outcomes, and the round holds the likeliest guess:
+//   - p below 1/2 acceptances a call: every step from the current position, as if each were
+//     rejected; the replay stops at the first acceptance;
+//   - p above 1/2: each in-bounds step from the one before it, as if each were accepted; the replay
+//     stops at the first rejection.
+// The depth is that of the batch retune, about 1.4 expected runs of the guess: 1.4 / p or
+// 1.4 / (1 - p), with the task's depth as the first estimate, worth 1.4 outcomes of the other kind.
+// A stand-alone walk has no batch before it: a fixed depth of 16 dropped 9 of 10 evaluations at
+// p = 0.6.  spec_cap 0 keeps the task's depth, over rejections: a depth fixed by the user, and the
+// sampler's walks, whose batch rule knows p (their own estimates, noisier, gained nothing).  Any choice gives the same
+// chain.  PAD4: rounds of a warp per proposal, padded to a multiple of four.  CH: compiled with the
+// look-ahead over acceptances.
+struct Round {
+  int depth;
+  bool chain;
+};
+template <bool PAD4, bool CH>
+__device__ __forceinline__ Round next_round(const WalkTask& T, int n_acc, int n_like) {
+  Round r;
+  r.depth = T.spec < 1 ? 1 : (T.spec > kSpecMax ? kSpecMax : T.spec);
+  r.chain = CH && T.spec_cap > 0 && 2 * n_acc > n_like;
   if (T.spec_cap > 0) {
-    m = (int)(1.4f * ((float)n_like + (float)m) / ((float)n_acc + 1.4f) + 0.5f);
-    m = min(max(m, 1), min(T.spec_cap, kSpecMax));
+    const int ends = r.chain ? n_like - n_acc : n_acc;
+    r.depth = (int)(1.4f * ((float)n_like + (float)r.depth) / ((float)ends + 1.4f) + 0.5f);
+    r.depth = min(max(r.depth, 1), min(T.spec_cap, kSpecMax));
   }
-  return PAD4 ? min((m + 3) & ~3, kSpecMax) : m;
+  if (PAD4) r.depth = min((r.depth + 3) & ~3, kSpecMax);
+  return r;
 }
 
 // ---------------------------------------------------------------- acceptance walk
@@ -721,13 +737,15 @@ __device__ __forceinline__ int round_depth(const WalkTask& T, int n_acc, int n_l
 // iff ln U < ln q(u) - ln q(u') (an independence Metropolis-Hastings test taken before the
 // likelihood); ln q of the current point is carried along and re-evaluated on CUDA cores
 // after an accepted DE move.
-template <int PREC, int NDET, int WF>
+template <int PREC, int NDET, int WF, bool CH>
 __global__ void __launch_bounds__(kThreads, 4) walk_kernel(const EventDev* __restrict__ evs, WalkTask* tasks,
                                                          const int32_t* __restrict__ blk_task,
                                                          const int32_t* __restrict__ blk_local) {
   constexpr int NV = NVals<NDET, WF>::value;
   __shared__ WalkerParams P[kSpecMax];
-  __shared__ SetupPart parts[kSpecMax];
+  __shared__ union { SetupPart parts[kSpecMax]; double diff[32][kMaxDim]; } sh;
+  SetupPart* const parts = sh.parts;
+  double (*const diff)[kMaxDim] = sh.diff;
   __shared__ double prop[kSpecMax][kMaxDim];
   __shared__ int cstep[kSpecMax];
   __shared__ int mstep[32];
@@ -737,7 +755,8 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel(const EventDev* __res
   __shared__ double u[kMaxDim];
   __shared__ float u32[kMaxDim];
   __shared__ int wcount[kWarps];
-  __shared__ int s_next, s_setup_warp, s_nin, s_end, s_needq, s_depth;
+  __shared__ int s_next, s_setup_warp, s_nin, s_end, s_needq;
+  __shared__ Round s_round;
   __shared__ int s_isflow[kSpecMax];
   __shared__ float s_lqf[kSpecMax];
   __shared__ float s_logq;
@@ -752,7 +771,6 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel(const EventDev* __res
   const uint64_t it = (uint64_t)T.iteration;
   const uint64_t wid = (uint64_t)(T.walker_offset + j);
   const uint64_t n_s = (uint64_t)T.n_s;
-  int m = round_depth<false>(T, 0, 0);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (threadIdx.x < D) {
     u[threadIdx.x] = T.u0[(size_t)j * D + threadIdx.x];
@@ -771,8 +789,9 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel(const EventDev* __res
   const float de_scale32 = (float)de_scale;
   __syncthreads();
   const int sw = s_setup_warp;
-  const bool use_flow = T.flow != nullptr && T.p_flow > 0.0;
+  const bool use_flow = !CH && T.flow != nullptr && T.p_flow > 0.0;
   const double p_flow = T.p_flow;
+  Round rd = next_round<false, CH>(T, 0, 0);
   if (use_flow) {
     const float lq = flow_logq_cta(*T.flow, u, fscr);
     if (threadIdx.x == 0) s_logq = lq;
@@ -781,6 +800,55 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel(const EventDev* __res
   int t = 0;
   while (t < n_steps) {
     const int abort_flag = threadIdx.x == 0 ? walk_abort_flag(T) : 0;
+    const int m = rd.depth;
+    if (CH && rd.chain) {
+      // 1. the setup warp forms the differences of the next 32 steps (a step a lane), then chains
+      //    the in-bounds moves (a coordinate a lane)
+      if (warp == sw) {
+        const int W = min(32, n_steps - t);
+        if (lane < W) {
+          const int st = t + lane;
+          Philox4 A = philox4x64((uint64_t)st, wid, it, 0ull, T.key0, T.key1);
+          const uint64_t a = rand_index(A.v[0], n_s);
+          uint64_t b = rand_index(A.v[1], n_s - 1);
+          b += (b >= a) ? 1ull : 0ull;
+          double sc = 1.0;
+          if ((A.v[2] >> 63) == 0ull) {
+            Philox4 B = philox4x64((uint64_t)st, wid, it, 1ull, T.key0, T.key1);
+            const double prod = __dmul_rn(__dmul_rn(__dmul_rn(rand_open_unit(B.v[0]), rand_open_unit(B.v[1])),
+                                                    rand_open_unit(B.v[2])), rand_open_unit(B.v[3]));
+            sc = __dmul_rn(de_scale, __dmul_rn(-0.25, log(prod)));
+          }
+          const double* ua = T.surv + a * D;
+          const double* ub = T.surv + b * D;
+#pragma unroll
+          for (int d = 0; d < kMaxDim; ++d)
+            if (d < D) diff[lane][d] = __dmul_rn(sc, __dsub_rn(ua[d], ub[d]));
+        }
+        __syncwarp();
+        const bool wrap = lane < D && ev.prior[ev.dim_param[lane]].periodic;
+        double x = lane < D ? u[lane] : 0.0;
+        int cnt = 0;
+        for (int q = 0; q < W && cnt < m; ++q) {
+          double y = 0.0;
+          if (lane < D) {
+            y = __dadd_rn(x, diff[q][lane]);
+            if (wrap) y = __dsub_rn(y, floor(y));
+          }
+          if (__all_sync(0xffffffffu, (unsigned long long)__double_as_longlong(y) <= 0x3FF0000000000000ull)) {
+            x = y;
+            if (lane < D) prop[cnt][lane] = y;
+            if (lane == 0) cstep[cnt] = t + q;
+            ++cnt;
+          }
+        }
+        __syncwarp();
+        if (lane == 0) {
+          s_nin = cnt;
+          s_end = cnt == m ? cstep[m - 1] : t + W - 1;
+        }
+      }
+    } else {
     const int W = min(min(kThreads, max(32, 4 * m)), n_steps - t);
     // 1a. every thread screens one candidate step in FP32
     int maybe = 0;
@@ -916,6 +984,7 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel(const EventDev* __res
       else end = t + W - 1;
       if (lane == 0) { s_nin = nin_w; s_end = end; }
     }
+    }
     __syncthreads();
     const int nin = s_nin;
     // 2. proposal constants on all four warps (setup_split.cuh), then the likelihoods: the sums of proposal i into tot_p[i] (chunk totals in ct), then one lane
@@ -952,23 +1021,30 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel(const EventDev* __res
     if (threadIdx.x == 0) {
       int nxt = s_end + 1;
       s_needq = 0;
+      int take = -1;   // the last accepted proposal
       for (int i = 0; i < nin; ++i) {
         ++n_like;
         n_bins += P[i].k_end;
-        if (lnl_p[i] > lnl_star) {
-          for (int d = 0; d < D; ++d) { u[d] = prop[i][d]; u32[d] = (float)prop[i][d]; }
-          lnl = lnl_p[i];
+        const bool up = lnl_p[i] > lnl_star;
+        if (up) {
+          take = i;
           ++n_acc;
+        }
+        if (up != (CH && rd.chain)) {   // the guess ends here
           nxt = cstep[i] + 1;
-          if (use_flow) {
-            if (s_isflow[i]) {
-              s_logq = s_lqf[i];
-              ++n_acc_flow;
-            } else {
-              s_needq = 1;
-            }
-          }
           break;
+        }
+      }
+      if (take >= 0) {
+        for (int d = 0; d < D; ++d) { u[d] = prop[take][d]; u32[d] = (float)prop[take][d]; }
+        lnl = lnl_p[take];
+        if (use_flow) {
+          if (s_isflow[take]) {
+            s_logq = s_lqf[take];
+            ++n_acc_flow;
+          } else {
+            s_needq = 1;
+          }
         }
       }
       n_spec += nin;
@@ -977,11 +1053,11 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel(const EventDev* __res
         if (T.status) atomicOr(T.status, 1);
       }
       s_next = nxt;
-      s_depth = round_depth<false>(T, n_acc, n_like);
+      s_round = next_round<false, CH>(T, n_acc, n_like);
     }
     __syncthreads();
     t = s_next;
-    m = s_depth;
+    rd = s_round;
     if (use_flow && s_needq && t < n_steps) {
       const float lq = flow_logq_cta(*T.flow, u, fscr);
       if (threadIdx.x == 0) s_logq = lq;
@@ -1036,14 +1112,19 @@ __device__ __forceinline__ ff ff_wrap_unit(ff x) {
 // phase takes as long for 1 or 5 proposals as for 4 or 8, and the padding only advances the
 // chain further.  The IMRPhenomD form (thousands of bins a proposal) runs each proposal on the
 // whole CTA instead.
-template <int NDET, int WF, bool XF>
+template <int NDET, int WF, bool XF, bool CH>
 __global__ void __launch_bounds__(kThreads, 4) walk_kernel_ff(const EventDev* __restrict__ evs, WalkTask* tasks,
                                                             const int32_t* __restrict__ blk_task,
                                                             const int32_t* __restrict__ blk_local) {
   constexpr int NV = NVals<NDET, WF>::value;
   __shared__ WalkerParams P[kSpecMax];
   __shared__ ff propf[kSpecMax][kMaxDim];
-  __shared__ std::conditional_t<WF == 0, TF2Part, PDPart> parts[kSpecMax];
+  __shared__ union Parts {
+    std::conditional_t<WF == 0, TF2Part, PDPart> p[kSpecMax];
+    ff diff[32][kMaxDim];
+    __device__ Parts() {}
+  } sh;
+  auto* const parts = sh.p;
   __shared__ int cstep[kSpecMax];
   __shared__ float part_sums[kSpecMax][2 * kMaxVals];
   __shared__ double s_rbl[kSpecMax];   // relative binning: ln L of each proposal
@@ -1054,7 +1135,8 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel_ff(const EventDev* __
   __shared__ double u[kMaxDim];
   __shared__ ff uf[kMaxDim];
   __shared__ int wcount[kWarps];
-  __shared__ int s_next, s_setup_warp, s_end, s_needq, s_depth;
+  __shared__ int s_next, s_setup_warp, s_end, s_needq, s_nin;
+  __shared__ Round s_round;
   __shared__ int s_isflow[kSpecMax];
   __shared__ float s_lqf[kSpecMax];
   __shared__ float s_logq;
@@ -1069,7 +1151,6 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel_ff(const EventDev* __
   const uint64_t it = (uint64_t)T.iteration;
   const uint64_t wid = (uint64_t)(T.walker_offset + j);
   const uint64_t n_s = (uint64_t)T.n_s;
-  int m = round_depth<WF == 0>(T, 0, 0);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const bool split = ev.ff_setup;
   if (threadIdx.x < D) {
@@ -1095,6 +1176,7 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel_ff(const EventDev* __
   const int sw = s_setup_warp;
   const bool use_flow = XF && T.flow != nullptr && T.p_flow > 0.0;
   const double p_flow = T.p_flow;
+  Round rd = next_round<WF == 0, CH>(T, 0, 0);
   if (use_flow) {
     const float lq = flow_logq_cta(*T.flow, u, fscr);
     if (threadIdx.x == 0) s_logq = lq;
@@ -1103,8 +1185,9 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel_ff(const EventDev* __
   int t = 0;
   while (t < n_steps) {
     const int abort_flag = threadIdx.x == 0 ? walk_abort_flag(T) : 0;
-    const int W = min(min(kThreads, max(32, 4 * m)), n_steps - t);
-    // 1. the exact move of one candidate step per thread
+    const int m = rd.depth, W = min((CH && rd.chain) ? 32 : min(kThreads, max(32, 4 * m)), n_steps - t);
+    // 1. the exact move of one candidate step per thread (looking ahead over acceptances: the
+    //    differences of the next 32 steps on warp 0, a step a lane)
     const int step = t + (int)threadIdx.x;
     int in = 0, isf = 0;
     float lqf = 0.0f;
@@ -1168,7 +1251,9 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel_ff(const EventDev* __
         in = 1;
 #pragma unroll
         for (int d = 0; d < kMaxDim; ++d) {
-          ff x = ff_add(uf[d < D ? d : D - 1], ff_mul(sc, ff_sub(ua[d], ub[d])));
+          const ff df = ff_mul(sc, ff_sub(ua[d], ub[d]));
+          if ((CH && rd.chain) && d < D) sh.diff[lane][d] = df;
+          ff x = ff_add(uf[d < D ? d : D - 1], df);
           const ff xw = ff_wrap_unit(x);
           if ((periodic >> d) & 1u) x = xw;
           if (d < D && !ff_in_unit(x)) in = 0;
@@ -1176,6 +1261,35 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel_ff(const EventDev* __
         }
       }
     }
+    int nin;
+    if (CH && rd.chain) {
+      // warp 0 chains the in-bounds moves, a coordinate a lane
+      if (warp == 0) {
+        __syncwarp();
+        ff x = lane < D ? uf[lane] : ff_make(0.0f);
+        int cnt = 0;
+        for (int q = 0; q < W && cnt < m; ++q) {
+          ff y = ff_make(0.0f);
+          if (lane < D) {
+            y = ff_add(x, sh.diff[q][lane]);
+            if ((periodic >> lane) & 1u) y = ff_wrap_unit(y);
+          }
+          if (__all_sync(0xffffffffu, ff_in_unit(y))) {
+            x = y;
+            if (lane < D) propf[cnt][lane] = y;
+            if (lane == 0) cstep[cnt] = t + q;
+            ++cnt;
+          }
+        }
+        __syncwarp();
+        if (lane == 0) {
+          s_nin = cnt;
+          s_end = cnt == m ? cstep[m - 1] : t + W - 1;
+        }
+      }
+      __syncthreads();
+      nin = s_nin;
+    } else {
     const unsigned mask = __ballot_sync(0xffffffffu, in);
     if (lane == 0) wcount[warp] = __popc(mask);
     __syncthreads();
@@ -1198,8 +1312,9 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel_ff(const EventDev* __
       if (slot == m - 1 && total > m) s_end = step;
     }
     if (threadIdx.x == 0 && total <= m) s_end = t + W - 1;
-    const int nin = min(total, m);
+    nin = min(total, m);
     __syncthreads();
+    }
     // 2. proposal constants
     if (nin > 0) {
       if (split) {
@@ -1229,8 +1344,10 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel_ff(const EventDev* __
     constexpr int V = Pow2Vals<NV>::value;
     constexpr int group = 32 / V;
     const bool rb = XF && ev.rb_nb > 0;
-    int neval = nin, pd_hit = -1;   // proposals evaluated; the accepted one (whole-CTA evaluations)
-    double pd_l = 0.0;
+    // whole-CTA evaluations: proposals evaluated, the last accepted one and its ln L, the one that
+    // ended the round's guess
+    int neval = nin, pd_hit = -1, pd_end = -1;
+    double pd_l = 0.0, pd_lnl = 0.0;
     if (rb) {
       // relative binning (~10^2 coarse-bin edges a proposal): a warp per proposal
       for (int i = warp; i < nin; i += kWarps) {
@@ -1272,7 +1389,15 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel_ff(const EventDev* __
         }
         neval = i + 1;
         pd_l = lnl_ff<NDET, WF>(ev, P[i], ps);
-        if (pd_l > lnl_star) { pd_hit = i; break; }
+        const bool up = pd_l > lnl_star;
+        if (up) {
+          pd_hit = i;
+          pd_lnl = pd_l;
+        }
+        if (up != (CH && rd.chain)) {
+          pd_end = i;
+          break;
+        }
       }
     } else {
       for (int i = warp; i < nin; i += kWarps) {
@@ -1298,14 +1423,24 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel_ff(const EventDev* __
           l = lnl_ff<NDET, WF>(ev, P[lane], part_sums[lane]);
         }
       }
+      // e: the proposal that ends the round's guess (its first acceptance, or first rejection);
+      // c: the last accepted one
       const unsigned am = __ballot_sync(0xffffffffu, lane < nin && l > lnl_star);
-      const int c = (WF == 1 && !rb) ? pd_hit : (am ? __ffs(am) - 1 : -1);
-      const int used = c >= 0 ? c + 1 : nin;
+      const unsigned live = nin < 32 ? (1u << nin) - 1u : 0xffffffffu;
+      const unsigned ends = ((CH && rd.chain) ? ~am : am) & live;
+      int e = ends ? __ffs(ends) - 1 : -1;
+      int c = (CH && rd.chain) ? (e >= 0 ? e : nin) - 1 : e;
+      if (WF == 1 && !rb) {
+        e = pd_end;
+        c = pd_hit;
+      }
+      const int used = e >= 0 ? e + 1 : nin;
+      const int acc = (CH && rd.chain) ? c + 1 : (c >= 0 ? 1 : 0);
       int kb = lane < used ? (rb ? s_rbk[lane] : P[lane].k_end) : 0;
 #pragma unroll
       for (int off = 16; off > 0; off >>= 1) kb += __shfl_xor_sync(0xffffffffu, kb, off);
       if (c >= 0) {
-        lnl = __shfl_sync(0xffffffffu, l, c);
+        lnl = (WF == 1 && !rb) ? pd_lnl : __shfl_sync(0xffffffffu, l, c);
         if (lane < D) {
           const ff x = propf[c][lane];
           uf[lane] = x;
@@ -1316,11 +1451,10 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel_ff(const EventDev* __
         n_like += used;
         n_bins += kb;
         n_spec += neval;
-        int nxt = s_end + 1;
+        int nxt = e >= 0 ? cstep[e] + 1 : s_end + 1;
         s_needq = 0;
+        n_acc += acc;
         if (c >= 0) {
-          ++n_acc;
-          nxt = cstep[c] + 1;
           if (use_flow) {
             if (s_isflow[c]) {
               s_logq = s_lqf[c];
@@ -1335,12 +1469,12 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel_ff(const EventDev* __
           if (T.status) atomicOr(T.status, 1);
         }
         s_next = nxt;
-        s_depth = round_depth<WF == 0>(T, n_acc, n_like);
+        s_round = next_round<WF == 0, CH>(T, n_acc, n_like);
       }
     }
     __syncthreads();
     t = s_next;
-    m = s_depth;
+    rd = s_round;
     if (use_flow && s_needq && t < n_steps) {
       const float lq = flow_logq_cta(*T.flow, u, fscr);
       if (threadIdx.x == 0) s_logq = lq;
@@ -1948,32 +2082,57 @@ cudaError_t launch_unit_likelihood_p(int waveform, int n_det, const EventDev* d_
   return cudaGetLastError();
 }
 
-// Mode 2 runs the float-float walk; modes 0 and 1 the FP64-recheck walk.  A launch whose tasks use neither flow proposals nor the relative-binning likelihood (extras false)
-// runs the float-float walk compiled without those paths (a smaller kernel: its round is
-// short and instruction fetch is among its first stalls).  Both properties of an event are
-// fixed before its first ns_step (ns_relbin_set is refused after it), so the sampler's
-// captured batch graphs keep a valid choice.
-template <int P, int N, int W>
-void launch_walk_one(int n_blocks, cudaStream_t s, const EventDev* d_evs, WalkTask* d_tasks,
-                     const int32_t* d_blk_task, const int32_t* d_blk_local, bool extras) {
-  if constexpr (P == 2) {
-    if (!extras)
-      walk_kernel_ff<N, W, false><<<n_blocks, kThreads, 0, s>>>(d_evs, d_tasks, d_blk_task, d_blk_local);
-    else
-      walk_kernel_ff<N, W, true><<<n_blocks, kThreads, 0, s>>>(d_evs, d_tasks, d_blk_task, d_blk_local);
-  } else {
-    walk_kernel<P, N, W><<<n_blocks, kThreads, 0, s>>>(d_evs, d_tasks, d_blk_task, d_blk_local);
+// Mode 2 runs the float-float walk; modes 0 and 1 the FP64-recheck walk.  A launch whose tasks use
+// neither flow proposals nor the relative-binning likelihood (extras false) runs the float-float
+// walk compiled without those paths (a smaller kernel: its round is short and instruction fetch is
+// among its first stalls).  Both properties of an event are fixed before its first ns_step
+// (ns_relbin_set is refused after it), so the sampler's captured batch graphs keep a valid choice.
+// `chain` launches (stand-alone walks) take the kernels that can look ahead over acceptances: their
+// acceptance may be anything (500 walkers x 600 steps at 0.87 acceptances a call, 4,017 bins: 4.85 ->
+// 2.1 ms).  The sampler's walks accept a few per cent of their calls from the first batches on, and
+// there the larger kernel costs 5 % (ten batches: 17.9 -> 19.0 ms of walks), so they take the plain
+// one; so do flows, and relative binning, which gained nothing (7.2 -> 7.5 ms).
+// The float-float walk's three variants are compiled in units of their own (GWNS_FF_WALK: parallel
+// builds).
+#define GWNS_WALK_ARGS \
+  int waveform, int n_det, const EventDev *d_evs, WalkTask *d_tasks, const int32_t *d_blk_task, \
+      const int32_t *d_blk_local, int n_blocks, cudaStream_t s
+cudaError_t launch_walk_ff_plain(GWNS_WALK_ARGS);    // kernels_p2w.cu
+cudaError_t launch_walk_ff_extras(GWNS_WALK_ARGS);   // kernels_p2.cu
+cudaError_t launch_walk_ff_chain(GWNS_WALK_ARGS);    // kernels_p2c.cu
+#define GWNS_FF_WALK(NAME, XF, CH)                                                                                   \
+  cudaError_t NAME(GWNS_WALK_ARGS) {                                                                                 \
+    GWNS_DISPATCH_W(GWNS_FF_WALK_ONE_##XF##CH, 2)                                                                    \
+    return cudaGetLastError();                                                                                       \
   }
+#define GWNS_FF_WALK_ONE_00(P_, N, W) \
+  walk_kernel_ff<N, W, false, false><<<n_blocks, kThreads, 0, s>>>(d_evs, d_tasks, d_blk_task, d_blk_local)
+#define GWNS_FF_WALK_ONE_10(P_, N, W) \
+  walk_kernel_ff<N, W, true, false><<<n_blocks, kThreads, 0, s>>>(d_evs, d_tasks, d_blk_task, d_blk_local)
+#define GWNS_FF_WALK_ONE_01(P_, N, W) \
+  walk_kernel_ff<N, W, false, true><<<n_blocks, kThreads, 0, s>>>(d_evs, d_tasks, d_blk_task, d_blk_local)
+
+template <int P, int N, int W>
+void launch_walk_f64(bool chain, int n_blocks, cudaStream_t s, const EventDev* d_evs, WalkTask* d_tasks,
+                     const int32_t* d_blk_task, const int32_t* d_blk_local) {
+  if (chain) walk_kernel<P, N, W, true><<<n_blocks, kThreads, 0, s>>>(d_evs, d_tasks, d_blk_task, d_blk_local);
+  else walk_kernel<P, N, W, false><<<n_blocks, kThreads, 0, s>>>(d_evs, d_tasks, d_blk_task, d_blk_local);
 }
 
 template <int P>
 cudaError_t launch_walk_p(int waveform, int n_det, const EventDev* d_evs, WalkTask* d_tasks,
                           const int32_t* d_blk_task, const int32_t* d_blk_local, int n_blocks, cudaStream_t s,
-                          bool extras) {
-#define GWNS_WALK(P_, N, W) launch_walk_one<P_, N, W>(n_blocks, s, d_evs, d_tasks, d_blk_task, d_blk_local, extras)
-  GWNS_DISPATCH_W(GWNS_WALK, P)
+                          bool extras, bool chain) {
+  if constexpr (P == 2) {
+    const auto f = extras ? launch_walk_ff_extras : chain ? launch_walk_ff_chain : launch_walk_ff_plain;
+    return f(waveform, n_det, d_evs, d_tasks, d_blk_task, d_blk_local, n_blocks, s);
+  } else {
+#define GWNS_WALK(P_, N, W) \
+  launch_walk_f64<P_, N, W>(chain && !extras, n_blocks, s, d_evs, d_tasks, d_blk_task, d_blk_local)
+    GWNS_DISPATCH_W(GWNS_WALK, P)
 #undef GWNS_WALK
-  return cudaGetLastError();
+    return cudaGetLastError();
+  }
 }
 
 // Mode 2 runs the speculative float-float HRSS kernel; modes 0 and 1 one candidate at a time.

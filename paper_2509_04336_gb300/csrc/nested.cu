@@ -480,7 +480,7 @@ int enqueue_batch(ns_handle* h, int b, int64_t* launches) {
                     h->n_walk_blocks, h->stream);
   } else {
     e = launch_walk(h->precision, h->waveform, h->max_det, h->d_events, h->d_tasks, h->d_blk_task, h->d_blk_local,
-                    h->n_walk_blocks, h->stream, walk_extras(h));
+                    h->n_walk_blocks, h->stream, walk_extras(h), false);
   }
   if (e != cudaSuccess) return cuda_fail(h, e, "walk launch");
   if ((e = cudaEventRecordWithFlags(h->walk_events[2 * b + 1], h->stream, cudaEventRecordExternal)) != cudaSuccess)
@@ -582,7 +582,6 @@ int nested_init(ns_handle* h) {
     std::memset(&T, 0, sizeof(T));
     T.surv = S.surv_u; T.survf = S.survf; T.u0 = S.w_u0; T.lnl0 = S.w_lnl0; T.u_out = S.w_uo; T.lnl_out = S.w_lo;
     T.n_acc = S.w_na; T.n_like = S.w_nl; T.n_bins = S.w_nb; T.n_spec = S.w_ns; T.spec = S.spec;
-    T.spec_cap = S.spec_auto ? S.spec_cap : 0;
     T.n_acc_flow = S.w_naf;
     T.lnl_star = -INFINITY; T.iteration = 0; T.walker_offset = 0;
     T.key0 = S.key0; T.key1 = S.key1; T.n_s = S.n_live - S.k; T.n = S.k; T.n_steps = S.n_steps;
@@ -680,8 +679,7 @@ int set_spec_cap(ns_handle* h, int cap) {
     cudaError_t err;
     if ((err = copy_on(h, &d->spec_cap, &cap, sizeof(int32_t), cudaMemcpyHostToDevice)) ||
         (err = copy_on(h, &d->spec, &spec, sizeof(int32_t), cudaMemcpyHostToDevice)) ||
-        (err = copy_on(h, &h->d_tasks[e].spec, &spec, sizeof(int32_t), cudaMemcpyHostToDevice)) ||
-        (err = copy_on(h, &h->d_tasks[e].spec_cap, &cap, sizeof(int32_t), cudaMemcpyHostToDevice)))
+        (err = copy_on(h, &h->d_tasks[e].spec, &spec, sizeof(int32_t), cudaMemcpyHostToDevice)))
       return cuda_fail(h, err, "speculation cap");
   }
   return NS_OK;
@@ -975,9 +973,7 @@ extern "C" int ns_state_load(ns_handle* h, const char* path) {
     std::memcpy(&S, &R.S, offsetof(NsState, live_u));
     S.dead_cap = E.ns.dead_cap;
     WalkTask* dt = h->d_tasks + e;
-    const int32_t task_cap = S.spec_auto ? S.spec_cap : 0;
     if ((err = copy_on(h, h->d_ns + e, &S, sizeof(S), cudaMemcpyHostToDevice)) ||
-        (err = copy_on(h, &dt->spec_cap, &task_cap, sizeof(int32_t), cudaMemcpyHostToDevice)) ||
         (err = copy_on(h, &dt->done, &S.done, sizeof(int32_t), cudaMemcpyHostToDevice)) ||
         (err = copy_on(h, &dt->n_steps, &S.n_steps, sizeof(int32_t), cudaMemcpyHostToDevice)) ||
         (err = copy_on(h, &dt->spec, &S.spec, sizeof(int32_t), cudaMemcpyHostToDevice)))
@@ -1067,7 +1063,7 @@ extern "C" int ns_batch_walk(ns_handle* h, int64_t walker_begin, int64_t walker_
   if ((e = cudaEventRecord(h->walk_events[0], h->stream)) != cudaSuccess) return cuda_fail(h, e, "event");
   e = h->hrss ? launch_hrss(h->precision, h->waveform, h->max_det, h->d_events, h->d_tasks, d_bt, d_bl, nb, h->stream)
               : launch_walk(h->precision, h->waveform, h->max_det, h->d_events, h->d_tasks, d_bt, d_bl, nb, h->stream,
-                            walk_extras(h));
+                            walk_extras(h), false);
   if (e != cudaSuccess) return cuda_fail(h, e, "walk launch");
   if ((e = cudaEventRecord(h->walk_events[1], h->stream)) != cudaSuccess) return cuda_fail(h, e, "event");
   if ((e = cudaStreamSynchronize(h->stream)) != cudaSuccess) return cuda_fail(h, e, "walk");
