@@ -36,10 +36,14 @@ constexpr uint32_t kBiasBytes = kBiasLayer * 4;   // 1152
 constexpr uint32_t kApWF0 = 0, kApWF1 = 45056, kApB0 = 90112, kApB1 = 91264, kApXA = 92416, kApHA = 96512;
 constexpr uint32_t kApBar = 129280;
 constexpr uint32_t kApBytes = kApBar + 64;
-// gradient kernel shared memory (bytes)
-constexpr uint32_t kGrXA = 0, kGrHA = 4096, kGrHB = 36864, kGrG3 = 69632, kGrWF = 77824, kGrW1T = 122880;
-constexpr uint32_t kGrW3T = 126976, kGrCS = 135168, kGrBias = 137216, kGrBar = 138368;
+// gradient kernel shared memory (bytes): two buffers of a layer's forward weights
+constexpr uint32_t kGrXA = 0, kGrHA = 4096, kGrHB = 36864, kGrG3 = 69632, kGrWF = 77824, kGrW1T = 167936;
+constexpr uint32_t kGrW3T = 172032, kGrCS = 180224, kGrBias = 182272, kGrBar = 183424;
 constexpr uint32_t kGrBytes = kGrBar + 64;
+// Threads of the gradient kernel: four groups of 128, group g on columns 32 g .. 32 g + 31 of every
+// hidden-layer epilogue.  A layer is a chain of MMA, commit, TMEM load, epilogue; with one group a
+// thread ran 128 tanh one after the other between two MMAs, and the tensor pipe was 4.6 % busy.
+constexpr int kGT = 512;
 static_assert(kGrBytes <= 232448, "gradient kernel shared memory");
 
 constexpr uint32_t kTmemCols = 256;
@@ -378,24 +382,29 @@ struct GradArgs {
   int32_t* err;
 };
 
-__global__ void __launch_bounds__(kFT, 1) flow_grad_kernel(GradArgs G) {
+__global__ void __launch_bounds__(kGT, 1) flow_grad_kernel(GradArgs G) {
   extern __shared__ __align__(1024) unsigned char sm[];
   if (G.active && *G.active == 0) return;
   FlowDev& F = *G.flow;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  // thread (r, grp): point r of the tile (row of the activations, TMEM lane), column group grp.  The
+  // point's state (z, g, ...) lives in group 0.  live: a warp whose rows hold points -- the images'
+  // other rows stay zero
+  const int r = tid & (kFT - 1), grp = tid / kFT, cg = 32 * grp;
+  const bool live = (warp & 3) * 32 < kGradRows;
   const int D = F.n_dim, L = F.n_layers, NP = F.n_params, LP = flow_layer_params(D);
   const int tile = blockIdx.x;
-  const int row = tile * kGradRows + tid;
-  const bool valid = tid < kGradRows && row < G.n;
+  const int row = tile * kGradRows + r;
+  const bool valid = grp == 0 && r < kGradRows && row < G.n;
   if (G.bump_t && tile == 0 && tid == 0) F.adam_t += 1;
 
   unsigned char *XA = sm + kGrXA, *HA = sm + kGrHA, *HB = sm + kGrHB, *G3 = sm + kGrG3;
-  unsigned char *WF = sm + kGrWF, *W1T = sm + kGrW1T, *W3T = sm + kGrW3T;
-  float* CS = reinterpret_cast<float*>(sm + kGrCS);             // [4 warps][128]
+  unsigned char *W1T = sm + kGrW1T, *W3T = sm + kGrW3T;
+  float* CS = reinterpret_cast<float*>(sm + kGrCS);             // [16 warps][32]
   float* bias = reinterpret_cast<float*>(sm + kGrBias);         // this layer's b1 | b2 | b3
-  uint64_t* bars = reinterpret_cast<uint64_t*>(sm + kGrBar);   // [0] weights, [1] W2T, [2] MMA
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + kGrBar + 32);
-  int* abort = reinterpret_cast<int*>(sm + kGrBar + 36);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(sm + kGrBar);   // [0], [1] weights, [2] MMA, [3] W2T, [4] W1T, W3T
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + kGrBar + 48);
+  int* abort = reinterpret_cast<int*>(sm + kGrBar + 52);
   float* part = G.partial + (size_t)tile * NP;
   float* zs = G.zsave + (size_t)tile * L * kFT * kFlowP;
 
@@ -404,29 +413,82 @@ __global__ void __launch_bounds__(kFT, 1) flow_grad_kernel(GradArgs G) {
     tc::tmem_relinquish();
   }
   if (tid == 0) {
-    for (int i = 0; i < 3; ++i) tc::mbar_init(&bars[i], 1);
+    for (int i = 0; i < 5; ++i) tc::mbar_init(&bars[i], 1);
     *abort = 0;
     tc::mbar_init_fence();
   }
+  for (uint32_t i = tid; i < kGrWF / 16; i += kGT) reinterpret_cast<uint4*>(sm)[i] = make_uint4(0u, 0u, 0u, 0u);
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
-  Tc T{*tslot, (uint32_t)(warp * 32) << 16, &bars[2], 0u, abort, 0, 0u};
-  uint32_t wpar = 0u, w2par = 0u;
-  int wpend = 0, w2pend = 0;
+  Tc T{*tslot, (uint32_t)((warp & 3) * 32) << 16, &bars[2], 0u, abort, 0, 0u};
+  // Weight copies, by thread 0: step s = 0 .. 2 L - 1 (forward layers, then backward) reads buffer
+  // s & 1; the copy of step s + 1 is issued when step s begins, so that it runs under step s
+  uint32_t wpar[2] = {0u, 0u}, w2par = 0u, wtpar = 0u;
+  int wpend[2] = {0, 0}, w2pend = 0, wtpend = 0;
+  auto layer_of = [&](int st) { return st < L ? st : 2 * L - 1 - st; };
+  auto issue = [&](int st) {
+    tc::mbar_expect_tx(&bars[st & 1], kImgFwd);
+    tc::bulk_g2s(sm + kGrWF + (st & 1) * kImgFwd, F.img + (size_t)layer_of(st) * kImgLayer, kImgFwd, &bars[st & 1]);
+    wpend[st & 1] = 1;
+  };
+  auto weights_in = [&](int st) {   // thread 0: false on timeout
+    if (!tc::mbar_wait(&bars[st & 1], wpar[st & 1])) return false;
+    wpar[st & 1] ^= 1u;
+    wpend[st & 1] = 0;
+    return true;
+  };
+  if (tid == 0) issue(0);
   bool ok = true;
 
-  // column sums of a [128 rows x 32 cols] block held one row per thread -> out[32]
-  auto colsum32 = [&](float* v, float* out) {
+  // column sums of the group's [128 rows x 32 cols] block held one row per thread; thread r < 32 of
+  // the group returns column r's
+  auto colsum32 = [&](float* v) {
     const float c = warp_colsum32(v, lane);
-    CS[warp * 128 + lane] = c;
+    CS[warp * 32 + lane] = c;
     __syncthreads();
-    if (tid < 32) out[tid] = CS[tid] + CS[128 + tid] + CS[256 + tid] + CS[384 + tid];
+    const float* q = CS + 4 * grp * 32 + lane;
+    const float t = q[0] + q[32] + q[64] + q[96];
     __syncthreads();
+    return t;
+  };
+  // tanh of the group's columns of G (+ bias) into an activation image
+  auto hidden = [&](unsigned char* img, const float* b) {
+    if (!live) return;
+#pragma unroll
+    for (int c0 = cg; c0 < cg + 32; c0 += 16) {
+      float v[16];
+      T.ld16(c0, v);
+#pragma unroll
+      for (int i = 0; i < 16; ++i) v[i] = flow_tanh(v[i] + b[c0 + i]);
+      st_row16(img, r, c0, v);
+    }
+  };
+  // gradient through the hidden layer in `img` (dh in TMEM columns 0 .. 127): the image becomes
+  // dh (1 - h^2), its column sums go to db
+  auto hidden_back = [&](unsigned char* img, float* db) {
+    float gp[32];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) gp[i] = 0.0f;
+    if (live) {
+      float h[16];
+      T.ld16(cg, gp);
+      T.ld16(cg + 16, gp + 16);
+      ld_row16(img, r, cg, h);
+#pragma unroll
+      for (int i = 0; i < 16; ++i) gp[i] *= 1.0f - h[i] * h[i];
+      ld_row16(img, r, cg + 16, h);
+#pragma unroll
+      for (int i = 0; i < 16; ++i) gp[16 + i] *= 1.0f - h[i] * h[i];
+      st_row16(img, r, cg, gp);
+      st_row16(img, r, cg + 16, gp + 16);
+    }
+    const float c = colsum32(gp);
+    if (r < 32) db[cg + r] = c;
   };
   // this layer's biases into shared memory (the previous readers passed a barrier)
   auto stage_bias = [&](int l) {
-    for (int i = tid; i < kBiasLayer; i += kFT) bias[i] = __ldg(F.bias + (size_t)l * kBiasLayer + i);
+    for (int i = tid; i < kBiasLayer; i += kGT) bias[i] = __ldg(F.bias + (size_t)l * kBiasLayer + i);
   };
 
   // ---- forward pass: layer inputs saved, log q for the loss
@@ -444,29 +506,26 @@ __global__ void __launch_bounds__(kFT, 1) flow_grad_kernel(GradArgs G) {
       }
   }
   for (int l = 0; l < L && ok; ++l) {
-    float4* zsl = reinterpret_cast<float4*>(zs + ((size_t)l * kFT + tid) * kFlowP);
+    unsigned char* WF = sm + kGrWF + (l & 1) * kImgFwd;
+    if (grp == 0) {
+      float4* zsl = reinterpret_cast<float4*>(zs + ((size_t)l * kFT + r) * kFlowP);
 #pragma unroll
-    for (int q = 0; q < 4; ++q) zsl[q] = make_float4(z[4 * q], z[4 * q + 1], z[4 * q + 2], z[4 * q + 3]);
-    if (tid == 0) {
-      tc::mbar_expect_tx(&bars[0], kImgFwd);
-      tc::bulk_g2s(WF, F.img + (size_t)l * kImgLayer, kImgFwd, &bars[0]);
-      wpend = 1;
+      for (int q = 0; q < 4; ++q) zsl[q] = make_float4(z[4 * q], z[4 * q + 1], z[4 * q + 2], z[4 * q + 3]);
     }
+    if (tid == 0) issue(l + 1);
     stage_bias(l);
-    {
+    if (grp == 0 && live) {
       float a[kFlowP];
 #pragma unroll
       for (int d = 0; d < kFlowP; ++d) a[d] = (d < D && flow_cond(l, d)) ? z[d] : 0.0f;
-      st_row16(XA, tid, 0, a);
+      st_row16(XA, r, 0, a);
     }
     Tc::publish();
     if (tid == 0) {
       tc::fence_after_sync();
-      if (!tc::mbar_wait(&bars[0], wpar)) {
+      if (!weights_in(l)) {
         *abort = 1;
       } else {
-        wpar ^= 1u;
-        wpend = 0;
         T.gemm(0, XA, WF + kImgW1, 128, 1);
         T.commit();
       }
@@ -474,14 +533,7 @@ __global__ void __launch_bounds__(kFT, 1) flow_grad_kernel(GradArgs G) {
     __syncthreads();
     if (*abort) { ok = false; break; }
     if (!(ok = T.wait())) break;
-#pragma unroll 1
-    for (int c0 = 0; c0 < kFlowH; c0 += 16) {
-      float v[16];
-      T.ld16(c0, v);
-#pragma unroll
-      for (int i = 0; i < 16; ++i) v[i] = flow_tanh(v[i] + bias[kBiasB1 + c0 + i]);
-      st_row16(HA, tid, c0, v);
-    }
+    hidden(HA, bias + kBiasB1);
     Tc::publish();
     if (tid == 0) {
       tc::fence_after_sync();
@@ -489,14 +541,7 @@ __global__ void __launch_bounds__(kFT, 1) flow_grad_kernel(GradArgs G) {
       T.commit();
     }
     if (!(ok = T.wait())) break;
-#pragma unroll 1
-    for (int c0 = 0; c0 < kFlowH; c0 += 16) {
-      float v[16];
-      T.ld16(c0, v);
-#pragma unroll
-      for (int i = 0; i < 16; ++i) v[i] = flow_tanh(v[i] + bias[kBiasB2 + c0 + i]);
-      st_row16(HB, tid, c0, v);
-    }
+    hidden(HB, bias + kBiasB2);
     Tc::publish();
     if (tid == 0) {
       tc::fence_after_sync();
@@ -504,7 +549,7 @@ __global__ void __launch_bounds__(kFT, 1) flow_grad_kernel(GradArgs G) {
       T.commit();
     }
     if (!(ok = T.wait())) break;
-    {
+    if (grp == 0 && live) {
       float sr[16], tt[16];
       T.ld16(128, sr);
       T.ld16(144, tt);
@@ -517,7 +562,7 @@ __global__ void __launch_bounds__(kFT, 1) flow_grad_kernel(GradArgs G) {
         }
     }
     tc::fence_before_sync();
-    __syncthreads();   // WF and the biases are reloaded by the next layer
+    __syncthreads();   // the other buffer and the biases are reloaded by the next layer
   }
   // loss part: sum over the tile's points of -log q
   float g[kFlowP];
@@ -530,7 +575,7 @@ __global__ void __launch_bounds__(kFT, 1) flow_grad_kernel(GradArgs G) {
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) nll += __shfl_xor_sync(0xffffffffu, nll, off);
-    if (lane == 0) CS[warp] = nll;
+    if (lane == 0 && grp == 0) CS[warp] = nll;
     __syncthreads();
     if (tid == 0) G.loss_part[tile] = (double)CS[0] + (double)CS[1] + (double)CS[2] + (double)CS[3];
     __syncthreads();
@@ -540,11 +585,13 @@ __global__ void __launch_bounds__(kFT, 1) flow_grad_kernel(GradArgs G) {
 
   // ---- backward pass
   for (int l = L - 1; l >= 0 && ok; --l) {
+    const int st = 2 * L - 1 - l;
+    unsigned char* WF = sm + kGrWF + (st & 1) * kImgFwd;
     const unsigned char* img = F.img + (size_t)l * kImgLayer;
     float* pl = part + (size_t)l * LP;
     float zin[kFlowP];
-    {
-      const float4* zsl = reinterpret_cast<const float4*>(zs + ((size_t)l * kFT + tid) * kFlowP);
+    if (grp == 0) {
+      const float4* zsl = reinterpret_cast<const float4*>(zs + ((size_t)l * kFT + r) * kFlowP);
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const float4 v = zsl[q];
@@ -552,27 +599,25 @@ __global__ void __launch_bounds__(kFT, 1) flow_grad_kernel(GradArgs G) {
       }
     }
     if (tid == 0) {
-      tc::mbar_expect_tx(&bars[0], kImgFwd + 4096 + 8192);
-      tc::bulk_g2s(WF, img, kImgFwd, &bars[0]);
-      tc::bulk_g2s(W1T, img + kImgW1T, 4096, &bars[0]);
-      tc::bulk_g2s(W3T, img + kImgW3T, 8192, &bars[0]);
-      wpend = 1;
+      if (st + 1 < 2 * L) issue(st + 1);
+      tc::mbar_expect_tx(&bars[4], 4096 + 8192);
+      tc::bulk_g2s(W1T, img + kImgW1T, 4096, &bars[4]);
+      tc::bulk_g2s(W3T, img + kImgW3T, 8192, &bars[4]);
+      wtpend = 1;
     }
     stage_bias(l);
-    {
+    if (grp == 0 && live) {
       float a[kFlowP];
 #pragma unroll
       for (int d = 0; d < kFlowP; ++d) a[d] = (d < D && flow_cond(l, d)) ? zin[d] : 0.0f;
-      st_row16(XA, tid, 0, a);
+      st_row16(XA, r, 0, a);
     }
     Tc::publish();
     if (tid == 0) {
       tc::fence_after_sync();
-      if (!tc::mbar_wait(&bars[0], wpar)) {
+      if (!weights_in(st)) {
         *abort = 1;
       } else {
-        wpar ^= 1u;
-        wpend = 0;
         T.gemm(0, XA, WF + kImgW1, 128, 1);
         T.commit();
       }
@@ -580,15 +625,7 @@ __global__ void __launch_bounds__(kFT, 1) flow_grad_kernel(GradArgs G) {
     __syncthreads();
     if (*abort) { ok = false; break; }
     if (!(ok = T.wait())) break;
-    // h1 -> HA
-#pragma unroll 1
-    for (int c0 = 0; c0 < kFlowH; c0 += 16) {
-      float v[16];
-      T.ld16(c0, v);
-#pragma unroll
-      for (int i = 0; i < 16; ++i) v[i] = flow_tanh(v[i] + bias[kBiasB1 + c0 + i]);
-      st_row16(HA, tid, c0, v);
-    }
+    hidden(HA, bias + kBiasB1);   // h1
     Tc::publish();
     if (tid == 0) {
       tc::fence_after_sync();
@@ -597,19 +634,11 @@ __global__ void __launch_bounds__(kFT, 1) flow_grad_kernel(GradArgs G) {
     }
     if (!(ok = T.wait())) break;
     if (tid == 0) {   // W2 has been consumed: bring W2T into its slot
-      tc::mbar_expect_tx(&bars[1], 32768);
-      tc::bulk_g2s(WF + kImgW2, img + kImgW2T, 32768, &bars[1]);
+      tc::mbar_expect_tx(&bars[3], 32768);
+      tc::bulk_g2s(WF + kImgW2, img + kImgW2T, 32768, &bars[3]);
       w2pend = 1;
     }
-    // h2 -> HB
-#pragma unroll 1
-    for (int c0 = 0; c0 < kFlowH; c0 += 16) {
-      float v[16];
-      T.ld16(c0, v);
-#pragma unroll
-      for (int i = 0; i < 16; ++i) v[i] = flow_tanh(v[i] + bias[kBiasB2 + c0 + i]);
-      st_row16(HB, tid, c0, v);
-    }
+    hidden(HB, bias + kBiasB2);   // h2
     Tc::publish();
     if (tid == 0) {
       tc::fence_after_sync();
@@ -619,78 +648,69 @@ __global__ void __launch_bounds__(kFT, 1) flow_grad_kernel(GradArgs G) {
     if (!(ok = T.wait())) break;
     // coupling backward: g_o = [d/ds_raw | d/dt] -> G3; db3; direct part of dz_in
     float gdir[kFlowP];
-    {
-      float sr[16], tt[16], go[32];
-      T.ld16(128, sr);
-      T.ld16(144, tt);
 #pragma unroll
-      for (int d = 0; d < kFlowP; ++d) {
-        go[d] = 0.0f;
-        go[16 + d] = 0.0f;
-        gdir[d] = g[d];
-        if (d < D && !flow_cond(l, d)) {
-          const float th = flow_tanh((sr[d] + bias[kBiasB3 + d]) / kFlowS);
-          const float e = expf(kFlowS * th);
-          const float gs = valid ? (g[d] * zin[d] * e - 1.0f) : 0.0f;
-          go[d] = gs * (1.0f - th * th);
-          go[16 + d] = g[d];
-          gdir[d] = g[d] * e;
+    for (int d = 0; d < kFlowP; ++d) gdir[d] = 0.0f;
+    {
+      float go[32];
+#pragma unroll
+      for (int i = 0; i < 32; ++i) go[i] = 0.0f;
+      if (grp == 0 && live) {
+        float sr[16], tt[16];
+        T.ld16(128, sr);
+        T.ld16(144, tt);
+#pragma unroll
+        for (int d = 0; d < kFlowP; ++d) {
+          gdir[d] = g[d];
+          if (d < D && !flow_cond(l, d)) {
+            const float th = flow_tanh((sr[d] + bias[kBiasB3 + d]) / kFlowS);
+            const float e = expf(kFlowS * th);
+            const float gs = valid ? (g[d] * zin[d] * e - 1.0f) : 0.0f;
+            go[d] = gs * (1.0f - th * th);
+            go[16 + d] = g[d];
+            gdir[d] = g[d] * e;
+          }
         }
+        st_row16(G3, r, 0, go);
+        st_row16(G3, r, 16, go + 16);
       }
-      st_row16(G3, tid, 0, go);
-      st_row16(G3, tid, 16, go + 16);
-      float cs[32];
-      colsum32(go, cs);   // go is consumed
+      const float c = colsum32(go);
       if (tid < kFlowO) {
         const int o = tid;
         const int op = o < 16 ? (o < D ? o : -1) : (o - 16 < D ? D + o - 16 : -1);
-        if (op >= 0) pl[flow_off_b3(D) + op] = cs[o];
+        if (op >= 0) pl[flow_off_b3(D) + op] = c;
       }
     }
     Tc::publish();
     if (tid == 0) {
       tc::fence_after_sync();
-      T.gemm(0, G3, W3T, 128, 2);         // dh2 = g_o W3
-      T.gemm_mn(128, HB, G3, 32, 8);      // dW3^T = h2^T g_o
-      T.commit();
+      if (!tc::mbar_wait(&bars[4], wtpar)) {
+        *abort = 1;
+      } else {
+        wtpar ^= 1u;
+        wtpend = 0;
+        T.gemm(0, G3, W3T, 128, 2);         // dh2 = g_o W3
+        T.gemm_mn(128, HB, G3, 32, 8);      // dW3^T = h2^T g_o
+        T.commit();
+      }
     }
+    __syncthreads();
+    if (*abort) { ok = false; break; }
     if (!(ok = T.wait())) break;
-    {
-      // dW3[o'][j] for hidden unit j = tid
+    if (grp < 2) {
+      // dW3[o'][j] for hidden unit j = r: outputs 16 grp ..
       float v[16];
-#pragma unroll 1
-      for (int c0 = 0; c0 < kFlowO; c0 += 16) {
-        T.ld16(128 + c0, v);
+      T.ld16(128 + 16 * grp, v);
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          const int o = c0 + i;
-          const int op = o < 16 ? (o < D ? o : -1) : (o - 16 < D ? D + o - 16 : -1);
-          if (op >= 0) pl[flow_off_w3(D) + op * kFlowH + tid] = v[i];
-        }
+      for (int i = 0; i < 16; ++i) {
+        const int op = i < D ? (grp == 0 ? i : D + i) : -1;
+        if (op >= 0) pl[flow_off_w3(D) + op * kFlowH + r] = v[i];
       }
     }
-    // g_p2 = dh2 (1 - h2^2) -> G2 over HB; db2
-#pragma unroll 1
-    for (int c0 = 0; c0 < kFlowH; c0 += 32) {
-      float gp[32], h[16];
-      T.ld16(c0, gp);
-      T.ld16(c0 + 16, gp + 16);
-      ld_row16(HB, tid, c0, h);
-#pragma unroll
-      for (int i = 0; i < 16; ++i) gp[i] *= 1.0f - h[i] * h[i];
-      ld_row16(HB, tid, c0 + 16, h);
-#pragma unroll
-      for (int i = 0; i < 16; ++i) gp[16 + i] *= 1.0f - h[i] * h[i];
-      st_row16(HB, tid, c0, gp);
-      st_row16(HB, tid, c0 + 16, gp + 16);
-      float cs[32];
-      colsum32(gp, cs);
-      if (tid < 32) pl[flow_off_b2(D) + c0 + tid] = cs[tid];
-    }
+    hidden_back(HB, pl + flow_off_b2(D));   // g_p2 = dh2 (1 - h2^2) over HB; db2
     Tc::publish();
     if (tid == 0) {
       tc::fence_after_sync();
-      if (!tc::mbar_wait(&bars[1], w2par)) {
+      if (!tc::mbar_wait(&bars[3], w2par)) {
         *abort = 1;
       } else {
         w2par ^= 1u;
@@ -704,34 +724,17 @@ __global__ void __launch_bounds__(kFT, 1) flow_grad_kernel(GradArgs G) {
     if (*abort) { ok = false; break; }
     if (!(ok = T.wait())) break;
     {
-      // dW2[j][k] for output unit j = tid
+      // dW2[j][k] for output unit j = r and the group's k, stored [k][j] (whole lines a warp; the
+      // rows of W2's own order are 512 bytes apart, 32 lines a store); flow_adam_kernel reads it so
       float v[16];
-#pragma unroll 1
-      for (int c0 = 0; c0 < kFlowH; c0 += 16) {
-        T.ld16(128 + c0, v);
-        float* dst = pl + flow_off_w2(D) + tid * kFlowH + c0;   // layer blocks are not 16-byte aligned
 #pragma unroll
-        for (int i = 0; i < 16; ++i) dst[i] = v[i];
+      for (int c0 = cg; c0 < cg + 32; c0 += 16) {
+        T.ld16(128 + c0, v);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) pl[flow_off_w2(D) + (c0 + i) * kFlowH + r] = v[i];
       }
     }
-    // g_p1 = dh1 (1 - h1^2) -> G1 over HA; db1
-#pragma unroll 1
-    for (int c0 = 0; c0 < kFlowH; c0 += 32) {
-      float gp[32], h[16];
-      T.ld16(c0, gp);
-      T.ld16(c0 + 16, gp + 16);
-      ld_row16(HA, tid, c0, h);
-#pragma unroll
-      for (int i = 0; i < 16; ++i) gp[i] *= 1.0f - h[i] * h[i];
-      ld_row16(HA, tid, c0 + 16, h);
-#pragma unroll
-      for (int i = 0; i < 16; ++i) gp[16 + i] *= 1.0f - h[i] * h[i];
-      st_row16(HA, tid, c0, gp);
-      st_row16(HA, tid, c0 + 16, gp + 16);
-      float cs[32];
-      colsum32(gp, cs);
-      if (tid < 32) pl[flow_off_b1(D) + c0 + tid] = cs[tid];
-    }
+    hidden_back(HA, pl + flow_off_b1(D));   // g_p1 = dh1 (1 - h1^2) over HA; db1
     Tc::publish();
     if (tid == 0) {
       tc::fence_after_sync();
@@ -740,22 +743,26 @@ __global__ void __launch_bounds__(kFT, 1) flow_grad_kernel(GradArgs G) {
       T.commit();
     }
     if (!(ok = T.wait())) break;
-    {
+    if (grp == 0) {
       float v[16];
-      T.ld16(192, v);   // dW1[j][d] for hidden unit j = tid
-#pragma unroll
-      for (int d = 0; d < kFlowP; ++d)
-        if (d < D) pl[tid * D + d] = v[d];
       T.ld16(128, v);   // g_a of this point
 #pragma unroll
       for (int d = 0; d < kFlowP; ++d) g[d] = gdir[d] + ((d < D && flow_cond(l, d)) ? v[d] : 0.0f);
+    } else if (grp == 1) {
+      float v[16];
+      T.ld16(192, v);   // dW1[j][d] for hidden unit j = r
+#pragma unroll
+      for (int d = 0; d < kFlowP; ++d)
+        if (d < D) pl[r * D + d] = v[d];
     }
     tc::fence_before_sync();
     __syncthreads();   // slots and biases are reloaded by the next layer
   }
   if (!ok && tid == 0) {
-    if (wpend) tc::mbar_wait(&bars[0], wpar);
-    if (w2pend) tc::mbar_wait(&bars[1], w2par);
+    for (int i = 0; i < 2; ++i)
+      if (wpend[i]) tc::mbar_wait(&bars[i], wpar[i]);
+    if (w2pend) tc::mbar_wait(&bars[3], w2par);
+    if (wtpend) tc::mbar_wait(&bars[4], wtpar);
     if (T.pend) tc::mbar_wait(&bars[2], T.pend_par);
     atomicExch(G.err, 1);
   }
@@ -815,9 +822,14 @@ __global__ void flow_adam_kernel(AdamArgs A) {
   const int NP = F.n_params;
   const float t = (float)F.adam_t;
   const float c1 = 1.0f / (1.0f - powf(0.9f, t)), c2 = 1.0f / (1.0f - powf(0.999f, t));
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < NP; i += gridDim.x * blockDim.x) {
+  const int D = F.n_dim, LP = flow_layer_params(D);
+  // q: place in the partial gradients, i: parameter (the partials hold W2's block transposed)
+  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < NP; q += gridDim.x * blockDim.x) {
     float gs = 0.0f;
-    for (int k = 0; k < A.n_tiles; ++k) gs += A.partial[(size_t)k * NP + i];
+    for (int k = 0; k < A.n_tiles; ++k) gs += A.partial[(size_t)k * NP + q];
+    const int l0 = q / LP * LP, w2 = q - l0 - flow_off_w2(D);
+    const int i = w2 >= 0 && w2 < kFlowH * kFlowH
+                      ? l0 + flow_off_w2(D) + (w2 % kFlowH) * kFlowH + w2 / kFlowH : q;
     const float g = gs * A.inv_n;
     if (A.grad_out) {
       A.grad_out[i] = g;
@@ -956,7 +968,7 @@ cudaError_t launch_flow_grad(FlowDev* d_flow, const double* d_u, int n, const in
                              float* d_partial, double* d_loss_part, float* d_zsave, int32_t* d_err, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   GradArgs G{d_flow, d_u, n, d_active, bump_t, d_partial, d_loss_part, d_zsave, d_err};
-  flow_grad_kernel<<<(n + kGradRows - 1) / kGradRows, kFT, kGrBytes, s>>>(G);
+  flow_grad_kernel<<<(n + kGradRows - 1) / kGradRows, kGT, kGrBytes, s>>>(G);
   return cudaGetLastError();
 }
 
