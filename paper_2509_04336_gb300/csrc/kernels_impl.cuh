@@ -9,6 +9,7 @@
 // compensation), then warp-shuffle trees (error-free two-sums in FP32) reduce them.
 #pragma once
 
+#include <cooperative_groups.h>
 #include <cstdio>
 #include <type_traits>
 
@@ -732,12 +733,13 @@ __device__ __forceinline__ Round next_round(const WalkTask& T, int n_acc, int n_
 // The chain, the accepted and likelihood-call counts and every ln L are those of the walk
 // that takes one step at a time.  The setup warp rotates over the CTAs of an SM (an arrival
 // counter), so their FP64 work lands on different sub-partitions.
+// CL: a cluster of CTAs per walker (launch_walk_f64).  CH: the look-ahead over acceptances.
 // Flow steps (task.flow set): a step whose Philox tag-6 draw falls below p_flow proposes the
 // precomputed flow sample of the proposal table instead of a DE move, and passes the screen
 // iff ln U < ln q(u) - ln q(u') (an independence Metropolis-Hastings test taken before the
 // likelihood); ln q of the current point is carried along and re-evaluated on CUDA cores
 // after an accepted DE move.
-template <int PREC, int NDET, int WF, bool CH>
+template <int PREC, int NDET, int WF, bool CH, bool CL>
 __global__ void __launch_bounds__(kThreads, 4) walk_kernel(const EventDev* __restrict__ evs, WalkTask* tasks,
                                                          const int32_t* __restrict__ blk_task,
                                                          const int32_t* __restrict__ blk_local) {
@@ -750,19 +752,24 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel(const EventDev* __res
   __shared__ int cstep[kSpecMax];
   __shared__ int mstep[32];
   __shared__ double lnl_p[kSpecMax];
-  __shared__ double tot_p[kSpecMax][NV];
+  __shared__ double tot_p[CL ? 2 : 1][kSpecMax][NV];   // by parity of the round: a rank ahead never overwrites
   __shared__ double ct[kWarps][kWarps][NV];
   __shared__ double u[kMaxDim];
   __shared__ float u32[kMaxDim];
   __shared__ int wcount[kWarps];
   __shared__ int s_next, s_setup_warp, s_nin, s_end, s_needq;
+  __shared__ int s_stop[2];
   __shared__ Round s_round;
   __shared__ int s_isflow[kSpecMax];
   __shared__ float s_lqf[kSpecMax];
   __shared__ float s_logq;
   __shared__ FlowScratch fscr;
-  const WalkTask& T = tasks[blk_task[blockIdx.x]];
-  const int j = blk_local[blockIdx.x];
+  // a walker's CTAs (a cluster; one CTA in large launches): every rank runs the same chain
+  namespace cg = cooperative_groups;
+  const cg::cluster_group cluster = cg::this_cluster();
+  const int ranks = CL ? (int)cluster.num_blocks() : 1, rank = CL ? (int)cluster.block_rank() : 0;
+  const WalkTask& T = tasks[blk_task[blockIdx.x / ranks]];
+  const int j = blk_local[blockIdx.x / ranks];
   const EventDev& ev = evs[T.event];
   if (T.done) return;
   const int D = ev.n_dim;
@@ -797,7 +804,7 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel(const EventDev* __res
     if (threadIdx.x == 0) s_logq = lq;
     __syncthreads();
   }
-  int t = 0;
+  int t = 0, par = 0;
   while (t < n_steps) {
     const int abort_flag = threadIdx.x == 0 ? walk_abort_flag(T) : 0;
     const int m = rd.depth;
@@ -995,27 +1002,43 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel(const EventDev* __res
       if (lane < nin) f64_split_second<PREC != 0, WF>(warp, ev, parts[lane], P[lane]);
       __syncthreads();
     }
-    if (nin >= kWarps) {
+    // proposals rank, rank + ranks, ... of the round; their totals go to every rank
+    const int mine = (nin - rank + ranks - 1) / ranks;
+    auto store_total = [&](int i, int q, double v) {
+      if (!CL) tot_p[par][i][q] = v;
+      else
+        for (int r = 0; r < ranks; ++r) *cluster.map_shared_rank(&tot_p[par][i][q], r) = v;
+    };
+    if (mine >= kWarps) {
       // one warp per proposal, its four chunks in turn
-      for (int i = warp; i < nin; i += kWarps) {
+      for (int i = rank + ranks * warp; i < nin; i += ranks * kWarps) {
         warp_chunks<PREC, NDET, WF>(ev, P[i], lane, ct[warp]);
-        if (lane < NV) tot_p[i][lane] = chunks_sum<NV>(ct[warp], lane);
+        if (lane < NV) store_total(i, lane, chunks_sum<NV>(ct[warp], lane));
         __syncwarp();
       }
     } else {
       // fewer proposals than warps: the whole CTA on each in turn, chunk w on warp w
-      for (int i = 0; i < nin; ++i) {
+      for (int i = rank; i < nin; i += ranks) {
         double dv[NV];
         float fv[NV], fc[NV];
         partials<PREC, NDET, WF>(ev, P[i], threadIdx.x, kThreads, dv, fv, fc);
         chunk_total<PREC, NV>(dv, fv, fc, lane, ct[0][warp]);
         __syncthreads();
-        if (threadIdx.x < NV) tot_p[i][threadIdx.x] = chunks_sum<NV>(ct[0], threadIdx.x);
+        if (threadIdx.x < NV) store_total(i, threadIdx.x, chunks_sum<NV>(ct[0], threadIdx.x));
         __syncthreads();
       }
     }
-    __syncthreads();
-    if (warp == sw && lane < nin) lnl_p[lane] = lnl_from_vals<PREC, NDET, WF>(ev, P[lane], tot_p[lane]);
+    if (CL) {
+      // rank 0 decides on the watchdog for all (each CTA has its own clock and view of the flag)
+      if (rank == 0 && threadIdx.x == 0) {
+        const int stop = walk_should_stop(T, t0, abort_flag) ? 1 : 0;
+        for (int r = 0; r < ranks; ++r) *cluster.map_shared_rank(&s_stop[par], r) = stop;
+      }
+      cluster.sync();
+    } else {
+      __syncthreads();
+    }
+    if (warp == sw && lane < nin) lnl_p[lane] = lnl_from_vals<PREC, NDET, WF>(ev, P[lane], tot_p[par][lane]);
     __syncthreads();
     // 3. the steps in order
     if (threadIdx.x == 0) {
@@ -1048,9 +1071,9 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel(const EventDev* __res
         }
       }
       n_spec += nin;
-      if (walk_should_stop(T, t0, abort_flag)) {   // watchdog: end the walk after this round
+      if (CL ? s_stop[par] != 0 : walk_should_stop(T, t0, abort_flag)) {   // watchdog: end the walk after this round
         nxt = n_steps;
-        if (T.status) atomicOr(T.status, 1);
+        if (T.status && rank == 0) atomicOr(T.status, 1);
       }
       s_next = nxt;
       s_round = next_round<false, CH>(T, n_acc, n_like);
@@ -1058,12 +1081,14 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel(const EventDev* __res
     __syncthreads();
     t = s_next;
     rd = s_round;
+    if (CL) par ^= 1;
     if (use_flow && s_needq && t < n_steps) {
       const float lq = flow_logq_cta(*T.flow, u, fscr);
       if (threadIdx.x == 0) s_logq = lq;
       __syncthreads();
     }
   }
+  if (rank != 0) return;
   if (threadIdx.x < D) T.u_out[(size_t)j * D + threadIdx.x] = u[threadIdx.x];
   if (threadIdx.x == 0) {
     T.lnl_out[j] = lnl;
@@ -2112,11 +2137,26 @@ cudaError_t launch_walk_ff_chain(GWNS_WALK_ARGS);    // kernels_p2c.cu
 #define GWNS_FF_WALK_ONE_01(P_, N, W) \
   walk_kernel_ff<N, W, false, true><<<n_blocks, kThreads, 0, s>>>(d_evs, d_tasks, d_blk_task, d_blk_local)
 
+// Modes 0 and 1 are bound by the FP64 pipe of a walker's SM (half of a round of eight proposals),
+// so a launch of few walkers spreads each over a cluster of CTAs: every rank runs the moves, the
+// constants and the replay, and evaluates its share of the round's proposals.
 template <int P, int N, int W>
-void launch_walk_f64(bool chain, int n_blocks, cudaStream_t s, const EventDev* d_evs, WalkTask* d_tasks,
+void launch_walk_f64(bool chain, int ranks, int n_blocks, cudaStream_t s, const EventDev* d_evs, WalkTask* d_tasks,
                      const int32_t* d_blk_task, const int32_t* d_blk_local) {
-  if (chain) walk_kernel<P, N, W, true><<<n_blocks, kThreads, 0, s>>>(d_evs, d_tasks, d_blk_task, d_blk_local);
-  else walk_kernel<P, N, W, false><<<n_blocks, kThreads, 0, s>>>(d_evs, d_tasks, d_blk_task, d_blk_local);
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = (unsigned)ranks;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(n_blocks * ranks));
+  cfg.blockDim = dim3(kThreads);
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = ranks > 1 ? 1 : 0;
+  // the error, if any, is read by the caller
+  const auto k = ranks > 1 ? (chain ? walk_kernel<P, N, W, true, true> : walk_kernel<P, N, W, false, true>)
+                           : (chain ? walk_kernel<P, N, W, true, false> : walk_kernel<P, N, W, false, false>);
+  cudaLaunchKernelEx(&cfg, k, d_evs, d_tasks, d_blk_task, d_blk_local);
 }
 
 template <int P>
@@ -2127,8 +2167,15 @@ cudaError_t launch_walk_p(int waveform, int n_det, const EventDev* d_evs, WalkTa
     const auto f = extras ? launch_walk_ff_extras : chain ? launch_walk_ff_chain : launch_walk_ff_plain;
     return f(waveform, n_det, d_evs, d_tasks, d_blk_task, d_blk_local, n_blocks, s);
   } else {
+    // the largest of 4, 2 and 1 ranks that gives every CTA an SM of its own (50 walkers of 1,969 bins,
+    // 26 batches to the evidence: 76 ms on one CTA each, 63 on two, 69 on three)
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    const int ranks = extras ? 1 : 4 * n_blocks <= sms ? 4 : 2 * n_blocks <= sms ? 2 : 1;
 #define GWNS_WALK(P_, N, W) \
-  launch_walk_f64<P_, N, W>(chain && !extras, n_blocks, s, d_evs, d_tasks, d_blk_task, d_blk_local)
+  launch_walk_f64<P_, N, W>(chain && !extras, ranks, n_blocks, s, d_evs, d_tasks, d_blk_task, d_blk_local)
     GWNS_DISPATCH_W(GWNS_WALK, P)
 #undef GWNS_WALK
     return cudaGetLastError();
