@@ -118,7 +118,7 @@ int flow_setup(ns_handle* h, int e) {
       (r = falloc(h, (void**)&Fh.d_v, sizeof(float) * NP, "adam v")) ||
       (r = falloc(h, (void**)&Fh.d_partial, sizeof(float) * NP * Fh.tiles_cap, "flow partial gradients")) ||
       (r = falloc(h, (void**)&Fh.d_loss_part, sizeof(double) * Fh.tiles_cap, "flow losses")) ||
-      (r = falloc(h, (void**)&Fh.d_zsave, sizeof(float) * Fh.tiles_cap * L * 128 * kFlowP, "flow layer inputs")) ||
+      (r = falloc(h, (void**)&Fh.d_zsave, sizeof(float) * Fh.tiles_cap * L * kGradSave, "flow activations")) ||
       (r = falloc(h, (void**)&Fh.d_grad, sizeof(float) * NP, "flow gradient")) ||
       (r = falloc(h, (void**)&Fh.d_tab_u, sizeof(double) * k * Fh.stride * D, "flow proposal table")) ||
       (r = falloc(h, (void**)&Fh.d_tab_lq, sizeof(double) * k * Fh.stride, "flow proposal table")) ||

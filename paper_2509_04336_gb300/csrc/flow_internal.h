@@ -13,6 +13,9 @@ namespace gwns {
 // rest are masked rows), so that twice as many CTAs share the survivors -- the kernel is bound by
 // its per-layer latency, not by the tensor pipe.
 constexpr int kGradRows = 64;
+// Floats the gradient kernel keeps of a (tile, layer) for its backward pass: the layer's inputs
+// [64][16], the bf16 rows of h1 and h2 (16 KB each), s_raw [64][16]
+constexpr int kGradSave = kGradRows * (16 + 64 + 64 + 16);
 
 // Device buffers of one event's flow (all owned by the handle).
 struct FlowHost {
@@ -27,7 +30,7 @@ struct FlowHost {
   float* d_v = nullptr;            // [n_params]
   float* d_partial = nullptr;      // [tiles_cap][n_params]
   double* d_loss_part = nullptr;   // [tiles_cap]
-  float* d_zsave = nullptr;        // [tiles_cap][L][128][16]
+  float* d_zsave = nullptr;        // [tiles_cap][L][kGradSave]
   float* d_grad = nullptr;         // [n_params] (gradient-only calls)
   int tiles_cap = 0;
   double* d_tab_u = nullptr;       // [k][stride][D] proposal table of the sampler's walks

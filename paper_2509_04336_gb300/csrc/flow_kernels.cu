@@ -13,8 +13,8 @@
 // Weights arrive by one bulk copy (cp.async.bulk) per layer, double-buffered in the apply
 // kernel so the next layer's copy overlaps this layer's work.
 //
-// The gradient kernel recomputes each layer's activations in the backward pass (from the
-// layer inputs it saved on the way forward) and forms, per tile,
+// The gradient kernel keeps each layer's inputs and activations on the way forward (40 KB a tile and
+// layer, written and read by the same CTA) and forms, per tile,
 //     dh2 = g_o W3,   dh1 = g_p2 W2,   g_a = g_p1 W1          (data gradients)
 //     dW3 = g_o^T h2, dW2 = g_p2^T h1, dW1 = g_p1^T a          (weight gradients, K = points)
 // all on the tensor cores, the weight gradients from transposed operand images written by
@@ -36,9 +36,10 @@ constexpr uint32_t kBiasBytes = kBiasLayer * 4;   // 1152
 constexpr uint32_t kApWF0 = 0, kApWF1 = 45056, kApB0 = 90112, kApB1 = 91264, kApXA = 92416, kApHA = 96512;
 constexpr uint32_t kApBar = 129280;
 constexpr uint32_t kApBytes = kApBar + 64;
-// gradient kernel shared memory (bytes): two buffers of a layer's forward weights
-constexpr uint32_t kGrXA = 0, kGrHA = 4096, kGrHB = 36864, kGrG3 = 69632, kGrWF = 77824, kGrW1T = 167936;
-constexpr uint32_t kGrW3T = 172032, kGrCS = 180224, kGrBias = 182272, kGrBar = 183424;
+// gradient kernel shared memory (bytes): two buffers of half a layer's weight images
+constexpr uint32_t kGrXA = 0, kGrHA = 4096, kGrHB = 36864, kGrG3 = 69632, kGrWF = 77824;
+constexpr uint32_t kGrCS = 167936, kGrBias = 169984, kGrBar = 171136;
+static_assert(kImgLayer == 2 * kImgFwd && kImgW1T == kImgFwd, "an image is its forward half, then its transposed half");
 constexpr uint32_t kGrBytes = kGrBar + 64;
 // Threads of the gradient kernel: four groups of 128, group g on columns 32 g .. 32 g + 31 of every
 // hidden-layer epilogue.  A layer is a chain of MMA, commit, TMEM load, epilogue; with one group a
@@ -378,7 +379,7 @@ struct GradArgs {
   int bump_t;              // advance Adam's step counter (training) or not (gradient only)
   float* partial;          // [n_tiles][n_params]
   double* loss_part;       // [n_tiles]
-  float* zsave;            // [n_tiles][L][128][16]
+  float* zsave;            // [n_tiles][L][kGradSave]
   int32_t* err;
 };
 
@@ -399,21 +400,20 @@ __global__ void __launch_bounds__(kGT, 1) flow_grad_kernel(GradArgs G) {
   if (G.bump_t && tile == 0 && tid == 0) F.adam_t += 1;
 
   unsigned char *XA = sm + kGrXA, *HA = sm + kGrHA, *HB = sm + kGrHB, *G3 = sm + kGrG3;
-  unsigned char *W1T = sm + kGrW1T, *W3T = sm + kGrW3T;
   float* CS = reinterpret_cast<float*>(sm + kGrCS);             // [16 warps][32]
   float* bias = reinterpret_cast<float*>(sm + kGrBias);         // this layer's b1 | b2 | b3
-  uint64_t* bars = reinterpret_cast<uint64_t*>(sm + kGrBar);   // [0], [1] weights, [2] MMA, [3] W2T, [4] W1T, W3T
+  uint64_t* bars = reinterpret_cast<uint64_t*>(sm + kGrBar);   // [0], [1] weights, [2] MMA
   uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + kGrBar + 48);
   int* abort = reinterpret_cast<int*>(sm + kGrBar + 52);
   float* part = G.partial + (size_t)tile * NP;
-  float* zs = G.zsave + (size_t)tile * L * kFT * kFlowP;
+  float* const save = G.zsave + (size_t)tile * L * kGradSave;
 
   if (warp == 0) {
     tc::tmem_alloc(tslot, kTmemCols);
     tc::tmem_relinquish();
   }
   if (tid == 0) {
-    for (int i = 0; i < 5; ++i) tc::mbar_init(&bars[i], 1);
+    for (int i = 0; i < 3; ++i) tc::mbar_init(&bars[i], 1);
     *abort = 0;
     tc::mbar_init_fence();
   }
@@ -423,13 +423,15 @@ __global__ void __launch_bounds__(kGT, 1) flow_grad_kernel(GradArgs G) {
   tc::fence_after_sync();
   Tc T{*tslot, (uint32_t)((warp & 3) * 32) << 16, &bars[2], 0u, abort, 0, 0u};
   // Weight copies, by thread 0: step s = 0 .. 2 L - 1 (forward layers, then backward) reads buffer
-  // s & 1; the copy of step s + 1 is issued when step s begins, so that it runs under step s
-  uint32_t wpar[2] = {0u, 0u}, w2par = 0u, wtpar = 0u;
-  int wpend[2] = {0, 0}, w2pend = 0, wtpend = 0;
+  // s & 1, a layer's forward images or its transposed ones; the copy of step s + 1 is issued when
+  // step s begins, so that it runs under step s
+  uint32_t wpar[2] = {0u, 0u};
+  int wpend[2] = {0, 0};
   auto layer_of = [&](int st) { return st < L ? st : 2 * L - 1 - st; };
   auto issue = [&](int st) {
     tc::mbar_expect_tx(&bars[st & 1], kImgFwd);
-    tc::bulk_g2s(sm + kGrWF + (st & 1) * kImgFwd, F.img + (size_t)layer_of(st) * kImgLayer, kImgFwd, &bars[st & 1]);
+    tc::bulk_g2s(sm + kGrWF + (st & 1) * kImgFwd, F.img + (size_t)layer_of(st) * kImgLayer + (st < L ? 0 : kImgFwd),
+                 kImgFwd, &bars[st & 1]);
     wpend[st & 1] = 1;
   };
   auto weights_in = [&](int st) {   // thread 0: false on timeout
@@ -452,8 +454,9 @@ __global__ void __launch_bounds__(kGT, 1) flow_grad_kernel(GradArgs G) {
     __syncthreads();
     return t;
   };
-  // tanh of the group's columns of G (+ bias) into an activation image
-  auto hidden = [&](unsigned char* img, const float* b) {
+  // tanh of the group's columns of G (+ bias) into an activation image and its copy `keep`
+  // ([16 chunks of 8 columns][64 rows], 16 bytes each) for the backward pass
+  auto hidden = [&](unsigned char* img, const float* b, uint4* keep) {
     if (!live) return;
 #pragma unroll
     for (int c0 = cg; c0 < cg + 32; c0 += 16) {
@@ -462,6 +465,9 @@ __global__ void __launch_bounds__(kGT, 1) flow_grad_kernel(GradArgs G) {
 #pragma unroll
       for (int i = 0; i < 16; ++i) v[i] = flow_tanh(v[i] + b[c0 + i]);
       st_row16(img, r, c0, v);
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+        keep[((c0 >> 3) + h) * kGradRows + r] = *reinterpret_cast<const uint4*>(img + tc::image_offset(128, r, c0 + 8 * h));
     }
   };
   // gradient through the hidden layer in `img` (dh in TMEM columns 0 .. 127): the image becomes
@@ -507,8 +513,10 @@ __global__ void __launch_bounds__(kGT, 1) flow_grad_kernel(GradArgs G) {
   }
   for (int l = 0; l < L && ok; ++l) {
     unsigned char* WF = sm + kGrWF + (l & 1) * kImgFwd;
-    if (grp == 0) {
-      float4* zsl = reinterpret_cast<float4*>(zs + ((size_t)l * kFT + r) * kFlowP);
+    float* const rec = save + (size_t)l * kGradSave;   // inputs | h1 | h2 | s_raw
+    uint4* const hrec = reinterpret_cast<uint4*>(rec + kGradRows * kFlowP);
+    if (grp == 0 && live) {
+      float4* zsl = reinterpret_cast<float4*>(rec + r * kFlowP);
 #pragma unroll
       for (int q = 0; q < 4; ++q) zsl[q] = make_float4(z[4 * q], z[4 * q + 1], z[4 * q + 2], z[4 * q + 3]);
     }
@@ -533,7 +541,7 @@ __global__ void __launch_bounds__(kGT, 1) flow_grad_kernel(GradArgs G) {
     __syncthreads();
     if (*abort) { ok = false; break; }
     if (!(ok = T.wait())) break;
-    hidden(HA, bias + kBiasB1);
+    hidden(HA, bias + kBiasB1, hrec);
     Tc::publish();
     if (tid == 0) {
       tc::fence_after_sync();
@@ -541,7 +549,7 @@ __global__ void __launch_bounds__(kGT, 1) flow_grad_kernel(GradArgs G) {
       T.commit();
     }
     if (!(ok = T.wait())) break;
-    hidden(HB, bias + kBiasB2);
+    hidden(HB, bias + kBiasB2, hrec + 16 * kGradRows);
     Tc::publish();
     if (tid == 0) {
       tc::fence_after_sync();
@@ -553,6 +561,9 @@ __global__ void __launch_bounds__(kGT, 1) flow_grad_kernel(GradArgs G) {
       float sr[16], tt[16];
       T.ld16(128, sr);
       T.ld16(144, tt);
+      float4* srec = reinterpret_cast<float4*>(hrec + 32 * kGradRows) + r * 4;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) srec[q] = make_float4(sr[4 * q], sr[4 * q + 1], sr[4 * q + 2], sr[4 * q + 3]);
 #pragma unroll
       for (int d = 0; d < kFlowP; ++d)
         if (d < D && !flow_cond(l, d)) {
@@ -583,69 +594,46 @@ __global__ void __launch_bounds__(kGT, 1) flow_grad_kernel(GradArgs G) {
 #pragma unroll
   for (int d = 0; d < kFlowP; ++d) g[d] = valid ? z[d] : 0.0f;
 
-  // ---- backward pass
+  // ---- backward pass: the activations as the forward pass left them (written by this CTA, ordered by
+  // its barriers), a layer's read ahead into registers
+  uint4 pf[4];
+  auto prefetch = [&](int l) {
+    const uint4* hrec = reinterpret_cast<const uint4*>(save + (size_t)l * kGradSave + kGradRows * kFlowP);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) pf[q] = hrec[tid + kGT * q];
+  };
+  if (ok) prefetch(L - 1);
   for (int l = L - 1; l >= 0 && ok; --l) {
     const int st = 2 * L - 1 - l;
-    unsigned char* WF = sm + kGrWF + (st & 1) * kImgFwd;
-    const unsigned char* img = F.img + (size_t)l * kImgLayer;
+    const unsigned char* WT = sm + kGrWF + (st & 1) * kImgFwd;   // W1T | W2T | W3T
+    const unsigned char *W1T = WT, *W2T = WT + (kImgW2T - kImgW1T), *W3T = WT + (kImgW3T - kImgW1T);
     float* pl = part + (size_t)l * LP;
-    float zin[kFlowP];
-    if (grp == 0) {
-      const float4* zsl = reinterpret_cast<const float4*>(zs + ((size_t)l * kFT + r) * kFlowP);
+    const float* const rec = save + (size_t)l * kGradSave;
+    float zin[kFlowP], sr[kFlowP];
+    if (grp == 0 && live) {
+      const float4* zsl = reinterpret_cast<const float4*>(rec + r * kFlowP);
+      const float4* ssl = reinterpret_cast<const float4*>(rec + kGradRows * (kFlowP + 128) + r * kFlowP);
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        const float4 v = zsl[q];
+        const float4 v = zsl[q], w = ssl[q];
         zin[4 * q] = v.x; zin[4 * q + 1] = v.y; zin[4 * q + 2] = v.z; zin[4 * q + 3] = v.w;
+        sr[4 * q] = w.x; sr[4 * q + 1] = w.y; sr[4 * q + 2] = w.z; sr[4 * q + 3] = w.w;
       }
     }
-    if (tid == 0) {
-      if (st + 1 < 2 * L) issue(st + 1);
-      tc::mbar_expect_tx(&bars[4], 4096 + 8192);
-      tc::bulk_g2s(W1T, img + kImgW1T, 4096, &bars[4]);
-      tc::bulk_g2s(W3T, img + kImgW3T, 8192, &bars[4]);
-      wtpend = 1;
-    }
+    if (tid == 0 && st + 1 < 2 * L) issue(st + 1);
     stage_bias(l);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {   // h1 -> HA, h2 -> HB
+      const int i = tid + kGT * q, c = (i & 1023) / kGradRows, row_ = i & (kGradRows - 1);
+      *reinterpret_cast<uint4*>((i < 1024 ? HA : HB) + tc::image_offset(128, row_, 8 * c)) = pf[q];
+    }
     if (grp == 0 && live) {
       float a[kFlowP];
 #pragma unroll
       for (int d = 0; d < kFlowP; ++d) a[d] = (d < D && flow_cond(l, d)) ? zin[d] : 0.0f;
       st_row16(XA, r, 0, a);
     }
-    Tc::publish();
-    if (tid == 0) {
-      tc::fence_after_sync();
-      if (!weights_in(st)) {
-        *abort = 1;
-      } else {
-        T.gemm(0, XA, WF + kImgW1, 128, 1);
-        T.commit();
-      }
-    }
-    __syncthreads();
-    if (*abort) { ok = false; break; }
-    if (!(ok = T.wait())) break;
-    hidden(HA, bias + kBiasB1);   // h1
-    Tc::publish();
-    if (tid == 0) {
-      tc::fence_after_sync();
-      T.gemm(0, HA, WF + kImgW2, 128, 8);
-      T.commit();
-    }
-    if (!(ok = T.wait())) break;
-    if (tid == 0) {   // W2 has been consumed: bring W2T into its slot
-      tc::mbar_expect_tx(&bars[3], 32768);
-      tc::bulk_g2s(WF + kImgW2, img + kImgW2T, 32768, &bars[3]);
-      w2pend = 1;
-    }
-    hidden(HB, bias + kBiasB2);   // h2
-    Tc::publish();
-    if (tid == 0) {
-      tc::fence_after_sync();
-      T.gemm(128, HB, WF + kImgW3, 32, 8);
-      T.commit();
-    }
-    if (!(ok = T.wait())) break;
+    __syncthreads();   // the biases
     // coupling backward: g_o = [d/ds_raw | d/dt] -> G3; db3; direct part of dz_in
     float gdir[kFlowP];
 #pragma unroll
@@ -655,9 +643,6 @@ __global__ void __launch_bounds__(kGT, 1) flow_grad_kernel(GradArgs G) {
 #pragma unroll
       for (int i = 0; i < 32; ++i) go[i] = 0.0f;
       if (grp == 0 && live) {
-        float sr[16], tt[16];
-        T.ld16(128, sr);
-        T.ld16(144, tt);
 #pragma unroll
         for (int d = 0; d < kFlowP; ++d) {
           gdir[d] = g[d];
@@ -683,11 +668,9 @@ __global__ void __launch_bounds__(kGT, 1) flow_grad_kernel(GradArgs G) {
     Tc::publish();
     if (tid == 0) {
       tc::fence_after_sync();
-      if (!tc::mbar_wait(&bars[4], wtpar)) {
+      if (!weights_in(st)) {
         *abort = 1;
       } else {
-        wtpar ^= 1u;
-        wtpend = 0;
         T.gemm(0, G3, W3T, 128, 2);         // dh2 = g_o W3
         T.gemm_mn(128, HB, G3, 32, 8);      // dW3^T = h2^T g_o
         T.commit();
@@ -710,18 +693,10 @@ __global__ void __launch_bounds__(kGT, 1) flow_grad_kernel(GradArgs G) {
     Tc::publish();
     if (tid == 0) {
       tc::fence_after_sync();
-      if (!tc::mbar_wait(&bars[3], w2par)) {
-        *abort = 1;
-      } else {
-        w2par ^= 1u;
-        w2pend = 0;
-        T.gemm(0, HB, WF + kImgW2, 128, 8);     // dh1 = g_p2 W2 (W2T image in the W2 slot)
-        T.gemm_mn(128, HB, HA, 128, 8);         // dW2 = g_p2^T h1
-        T.commit();
-      }
+      T.gemm(0, HB, W2T, 128, 8);       // dh1 = g_p2 W2
+      T.gemm_mn(128, HB, HA, 128, 8);   // dW2 = g_p2^T h1
+      T.commit();
     }
-    __syncthreads();
-    if (*abort) { ok = false; break; }
     if (!(ok = T.wait())) break;
     {
       // dW2[j][k] for output unit j = r and the group's k, stored [k][j] (whole lines a warp; the
@@ -742,6 +717,7 @@ __global__ void __launch_bounds__(kGT, 1) flow_grad_kernel(GradArgs G) {
       T.gemm_mn(192, HA, XA, 16, 8);     // dW1 = g_p1^T a
       T.commit();
     }
+    if (l > 0) prefetch(l - 1);
     if (!(ok = T.wait())) break;
     if (grp == 0) {
       float v[16];
@@ -761,8 +737,6 @@ __global__ void __launch_bounds__(kGT, 1) flow_grad_kernel(GradArgs G) {
   if (!ok && tid == 0) {
     for (int i = 0; i < 2; ++i)
       if (wpend[i]) tc::mbar_wait(&bars[i], wpar[i]);
-    if (w2pend) tc::mbar_wait(&bars[3], w2par);
-    if (wtpend) tc::mbar_wait(&bars[4], wtpar);
     if (T.pend) tc::mbar_wait(&bars[2], T.pend_par);
     atomicExch(G.err, 1);
   }
@@ -826,7 +800,16 @@ __global__ void flow_adam_kernel(AdamArgs A) {
   // q: place in the partial gradients, i: parameter (the partials hold W2's block transposed)
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < NP; q += gridDim.x * blockDim.x) {
     float gs = 0.0f;
-    for (int k = 0; k < A.n_tiles; ++k) gs += A.partial[(size_t)k * NP + q];
+    // eight loads in flight (the sum stays in tile order)
+    int k = 0;
+    for (; k + 8 <= A.n_tiles; k += 8) {
+      float v[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) v[j] = A.partial[(size_t)(k + j) * NP + q];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) gs += v[j];
+    }
+    for (; k < A.n_tiles; ++k) gs += A.partial[(size_t)k * NP + q];
     const int l0 = q / LP * LP, w2 = q - l0 - flow_off_w2(D);
     const int i = w2 >= 0 && w2 < kFlowH * kFlowH
                       ? l0 + flow_off_w2(D) + (w2 % kFlowH) * kFlowH + w2 / kFlowH : q;
