@@ -792,22 +792,19 @@ extern "C" int ns_step(ns_handle* h, int max_batches, ns_progress* progress) {
   return warn ? NS_WMAXMCMC : NS_OK;
 }
 
-extern "C" int ns_evidence(ns_handle* h, int event, double* log_z, double* log_z_err, double* info_h,
-                           int64_t* n_like) {
-  if (!h) return set_error(nullptr, NS_EINVAL, "handle is NULL");
-  if (event < 0 || event >= (int)h->events.size()) return set_error(h, NS_EINVAL, "event out of range");
-  cudaSetDevice(h->device);
+// ln Z of an event and (info_h not null) its information H from the current state, in FP64:
+// ln Z = logsumexp(dead ln w, live ln L + ln X - ln n).
+static int evidence_sums(ns_handle* h, int event, double* log_z, double* info_h) {
   int r = download_states(h);
   if (r) return r;
   const NsState& S = h->host_ns[event];
   const int64_t nd = S.n_dead;
-  std::vector<double> dl(nd), dw(nd), ll(S.n_live);
+  std::vector<double> dl(info_h ? nd : 0), dw(nd), ll(S.n_live);
   cudaError_t e;
-  if ((e = copy_on(h, dl.data(), S.dead_lnl, sizeof(double) * nd, cudaMemcpyDeviceToHost)) ||
+  if ((info_h && (e = copy_on(h, dl.data(), S.dead_lnl, sizeof(double) * nd, cudaMemcpyDeviceToHost))) ||
       (e = copy_on(h, dw.data(), S.dead_logw, sizeof(double) * nd, cudaMemcpyDeviceToHost)) ||
       (e = copy_on(h, ll.data(), S.live_lnl, sizeof(double) * S.n_live, cudaMemcpyDeviceToHost)))
     return cuda_fail(h, e, "evidence download");
-  // ln Z = logsumexp(dead ln w, live ln L + ln X - ln n), in FP64
   double m = -INFINITY;
   for (double v : dw) m = std::fmax(m, v);
   const double lxn = S.log_x - std::log((double)S.n_live);
@@ -816,9 +813,26 @@ extern "C" int ns_evidence(ns_handle* h, int event, double* log_z, double* log_z
   for (double v : dw) s += std::exp(v - m);
   for (double v : ll) s += std::exp(v + lxn - m);
   const double lz = m + std::log(s);
-  double hsum = 0.0;
-  for (int64_t i = 0; i < nd; ++i) hsum += std::exp(dw[i] - lz) * dl[i];
-  for (double v : ll) hsum += std::exp(v + lxn - lz) * v;
+  if (info_h) {
+    double hsum = 0.0;
+    for (int64_t i = 0; i < nd; ++i) hsum += std::exp(dw[i] - lz) * dl[i];
+    for (double v : ll) hsum += std::exp(v + lxn - lz) * v;
+    *info_h = hsum - lz;
+  }
+  *log_z = lz;
+  return NS_OK;
+}
+
+extern "C" int ns_evidence(ns_handle* h, int event, double* log_z, double* log_z_err, double* info_h,
+                           int64_t* n_like) {
+  if (!h) return set_error(nullptr, NS_EINVAL, "handle is NULL");
+  if (event < 0 || event >= (int)h->events.size()) return set_error(h, NS_EINVAL, "event out of range");
+  cudaSetDevice(h->device);
+  double lz, info;
+  int r = evidence_sums(h, event, &lz, &info);
+  if (r) return r;
+  const NsState& S = h->host_ns[event];
+  cudaError_t e;
   // replays on the device
   const int R = 200;
   double* d_out;
@@ -837,7 +851,7 @@ extern "C" int ns_evidence(ns_handle* h, int event, double* log_z, double* log_z
   for (double v : rep) var += (v - mean) * (v - mean);
   if (log_z) *log_z = lz;
   if (log_z_err) *log_z_err = std::sqrt(var / R);
-  if (info_h) *info_h = hsum - lz;
+  if (info_h) *info_h = info;
   if (n_like) *n_like = S.n_like;
   return NS_OK;
 }
@@ -848,14 +862,15 @@ extern "C" int ns_posterior(ns_handle* h, int event, double* theta_out, double* 
   if (event < 0 || event >= (int)h->events.size()) return set_error(h, NS_EINVAL, "event out of range");
   if (cap < 0 || (cap > 0 && (!theta_out || !logw_out))) return set_error(h, NS_EINVAL, "bad output arrays");
   cudaSetDevice(h->device);
-  double lz;
-  int r = ns_evidence(h, event, &lz, nullptr, nullptr, nullptr);
+  int r = download_states(h);
   if (r) return r;
   const NsState& S = h->host_ns[event];
   const int64_t total = S.n_dead + S.n_live;
   if (n_out) *n_out = total;
   const int64_t m = cap < total ? cap : total;
-  if (m == 0) return NS_OK;
+  if (m == 0) return NS_OK;   // the count alone, as a caller asks for it before it allocates
+  double lz;
+  if ((r = evidence_sums(h, event, &lz, nullptr))) return r;
   const int D = S.D;
   double *d_u, *d_th;
   if ((r = alloc(h, (void**)&d_u, sizeof(double) * m * D, "posterior u"))) return r;
