@@ -1160,6 +1160,10 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel_ff(const EventDev* __
   __shared__ double u[kMaxDim];
   __shared__ ff uf[kMaxDim];
   __shared__ int wcount[kWarps];
+  __shared__ unsigned wmask[kWarps];
+  // candidates of a round: the step (complemented: unit scale), its survivors, the scale's uniforms
+  __shared__ int cand_step[XF ? 1 : 32], cand_a[XF ? 1 : 32], cand_b[XF ? 1 : 32];
+  __shared__ uint64_t cand_u[XF ? 1 : 32][4];
   __shared__ int s_next, s_setup_warp, s_end, s_needq, s_nin;
   __shared__ Round s_round;
   __shared__ int s_isflow[kSpecMax];
@@ -1210,9 +1214,173 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel_ff(const EventDev* __
   int t = 0;
   while (t < n_steps) {
     const int abort_flag = threadIdx.x == 0 ? walk_abort_flag(T) : 0;
-    const int m = rd.depth, W = min((CH && rd.chain) ? 32 : min(kThreads, max(32, 4 * m)), n_steps - t);
-    // 1. the exact move of one candidate step per thread (looking ahead over acceptances: the
-    //    differences of the next 32 steps on warp 0, a step a lane)
+    const int m = rd.depth;
+    int nin;
+    if constexpr (!XF) {
+      // 1a. one step a thread: its draws and, looking ahead over rejections, a FP32 screen of its move
+      //     (as in walk_kernel: the margin never rejects a step that the exact test accepts).  Four
+      //     moves of five leave the cube, and the exact move of one is ~700 float-float
+      //     instructions: it is formed for the steps that may stay only.  Looking ahead over
+      //     acceptances: the next 32 steps, unscreened.
+      const bool chain = CH && rd.chain;
+      const int W = min(chain ? 32 : min(kThreads, max(32, 4 * m)), n_steps - t);
+      const int step = t + (int)threadIdx.x;
+      int maybe = 0, ia = 0, ib = 0;
+      bool draw_scale = false;
+      Philox4 B;
+      if ((int)threadIdx.x < W) {
+        // tag 0: survivors and scale coin, tag 1: the scale's uniforms -- one inlined generator
+        Philox4 A;
+#pragma unroll 1
+        for (int tag = 0; tag < 2; ++tag) {
+          const Philox4 r = philox4x64((uint64_t)step, wid, it, (uint64_t)tag, T.key0, T.key1);
+          if (tag == 0) {
+            A = r;
+            draw_scale = (r.v[2] >> 63) == 0ull;
+            if (!draw_scale) break;
+          } else {
+            B = r;
+          }
+        }
+        ia = (int)rand_index(A.v[0], n_s);
+        ib = (int)rand_index(A.v[1], n_s - 1);
+        ib += ib >= ia ? 1 : 0;
+        maybe = 1;
+        if (!chain) {
+          float va[kMaxDim], vb[kMaxDim];   // both survivors first: all loads in flight at once
+#pragma unroll
+          for (int d = 0; d < kMaxDim; ++d) {
+            const size_t dd = d < D ? d : D - 1;
+            va[d] = T.survf ? T.survf[(size_t)ia * D + dd].x : (float)T.surv[(size_t)ia * D + dd];
+            vb[d] = T.survf ? T.survf[(size_t)ib * D + dd].x : (float)T.surv[(size_t)ib * D + dd];
+          }
+          float sc = 1.0f;
+          if (draw_scale) {
+            const float l2 = __log2f(top52_half_f(B.v[0])) + __log2f(top52_half_f(B.v[1])) +
+                             __log2f(top52_half_f(B.v[2])) + __log2f(top52_half_f(B.v[3])) - 208.0f;
+            sc = de_scale.h * (-0.25f * 0.6931471805599453f * l2);
+          }
+          const float margin = 1e-5f * (1.0f + fabsf(sc));
+#pragma unroll
+          for (int d = 0; d < kMaxDim; ++d) {
+            const float x = uf[d < D ? d : D - 1].h + sc * (va[d] - vb[d]);
+            if (d < D && !((periodic >> d) & 1u) && !(x >= -margin && x <= 1.0f + margin)) maybe = 0;
+          }
+        }
+      }
+      const unsigned mask = __ballot_sync(0xffffffffu, maybe);
+      if (lane == 0) wcount[warp] = __popc(mask);
+      __syncthreads();
+      int before = 0, total = 0;
+#pragma unroll
+      for (int w2 = 0; w2 < kWarps; ++w2) {
+        const int cw = wcount[w2];
+        before += (w2 < warp) ? cw : 0;
+        total += cw;
+      }
+      const int cs = before + __popc(mask & ((1u << lane) - 1u));
+      if (maybe && cs < 32) {
+        cand_step[cs] = draw_scale ? step : ~step;
+        cand_a[cs] = ia;
+        cand_b[cs] = ib;
+        if (draw_scale) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) cand_u[cs][q] = B.v[q];
+        }
+      }
+      const int nc = min(total, 32);
+      __syncthreads();
+      // 1b. the exact moves: candidate `lane`, coordinates warp, warp + 4, ... (float-float)
+      constexpr int kQ = (kMaxDim + kWarps - 1) / kWarps;
+      ff xq[kQ];
+      int in = lane < nc;
+      int st = 0;
+      if (lane < nc) {
+        st = cand_step[lane];
+        ff sc = ff_make(1.0f);
+        if (st >= 0) sc = ff_mul(ff_mul_f(ff_log_uniform_product(cand_u[lane]), -0.25f), de_scale);
+        else st = ~st;
+        const size_t oa = (size_t)cand_a[lane] * D, ob = (size_t)cand_b[lane] * D;
+        ff ua[kQ], ub[kQ];
+#pragma unroll
+        for (int q = 0; q < kQ; ++q) {
+          const int d = min(warp + kWarps * q, D - 1);
+          if (T.survf) {
+            const float2 pa = T.survf[oa + d], pb = T.survf[ob + d];
+            ua[q] = ff{pa.x, pa.y};
+            ub[q] = ff{pb.x, pb.y};
+          } else {
+            ua[q] = ff_from_double(T.surv[oa + d]);
+            ub[q] = ff_from_double(T.surv[ob + d]);
+          }
+        }
+#pragma unroll
+        for (int q = 0; q < kQ; ++q) {
+          const int d = warp + kWarps * q;
+          if (d < D) {
+            const ff df = ff_mul(sc, ff_sub(ua[q], ub[q]));
+            if (chain) {
+              sh.diff[lane][d] = df;
+            } else {
+              ff x = ff_add(uf[d], df);
+              if ((periodic >> d) & 1u) x = ff_wrap_unit(x);
+              if (!ff_in_unit(x)) in = 0;
+              xq[q] = x;
+            }
+          }
+        }
+      }
+      if (!chain) {
+        const unsigned mine = __ballot_sync(0xffffffffu, in);
+        if (lane == 0) wmask[warp] = mine;
+        __syncthreads();
+        const unsigned im = wmask[0] & wmask[1] & wmask[2] & wmask[3];
+        const int cnt = __popc(im), slot = __popc(im & ((1u << lane) - 1u));
+        if (((im >> lane) & 1u) && slot < m) {
+#pragma unroll
+          for (int q = 0; q < kQ; ++q)
+            if (warp + kWarps * q < D) propf[slot][warp + kWarps * q] = xq[q];
+          if (warp == 0) {
+            cstep[slot] = st;
+            // the round covers the steps up to the m-th in-bounds one, else the last candidate if
+            // there were more than 32, else the whole window
+            if (slot == m - 1 && cnt > m) s_end = st;
+          }
+        }
+        if (threadIdx.x == 31 && cnt <= m) s_end = total > 32 ? st : t + W - 1;
+        nin = min(cnt, m);
+        __syncthreads();
+      } else {
+        // warp 0 chains the in-bounds moves, a coordinate a lane
+        __syncthreads();
+        if (warp == 0) {
+          ff x = lane < D ? uf[lane] : ff_make(0.0f);
+          int cnt = 0;
+          for (int q = 0; q < W && cnt < m; ++q) {
+            ff y = ff_make(0.0f);
+            if (lane < D) {
+              y = ff_add(x, sh.diff[q][lane]);
+              if ((periodic >> lane) & 1u) y = ff_wrap_unit(y);
+            }
+            if (__all_sync(0xffffffffu, ff_in_unit(y))) {
+              x = y;
+              if (lane < D) propf[cnt][lane] = y;
+              if (lane == 0) cstep[cnt] = t + q;
+              ++cnt;
+            }
+          }
+          __syncwarp();
+          if (lane == 0) {
+            s_nin = cnt;
+            s_end = cnt == m ? cstep[m - 1] : t + W - 1;
+          }
+        }
+        __syncthreads();
+        nin = s_nin;
+      }
+    } else {
+      // 1. flow proposals or relative binning: the exact move of one candidate step per thread
+      const int W = min(min(kThreads, max(32, 4 * m)), n_steps - t);
     const int step = t + (int)threadIdx.x;
     int in = 0, isf = 0;
     float lqf = 0.0f;
@@ -1277,7 +1445,6 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel_ff(const EventDev* __
 #pragma unroll
         for (int d = 0; d < kMaxDim; ++d) {
           const ff df = ff_mul(sc, ff_sub(ua[d], ub[d]));
-          if ((CH && rd.chain) && d < D) sh.diff[lane][d] = df;
           ff x = ff_add(uf[d < D ? d : D - 1], df);
           const ff xw = ff_wrap_unit(x);
           if ((periodic >> d) & 1u) x = xw;
@@ -1286,35 +1453,6 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel_ff(const EventDev* __
         }
       }
     }
-    int nin;
-    if (CH && rd.chain) {
-      // warp 0 chains the in-bounds moves, a coordinate a lane
-      if (warp == 0) {
-        __syncwarp();
-        ff x = lane < D ? uf[lane] : ff_make(0.0f);
-        int cnt = 0;
-        for (int q = 0; q < W && cnt < m; ++q) {
-          ff y = ff_make(0.0f);
-          if (lane < D) {
-            y = ff_add(x, sh.diff[q][lane]);
-            if ((periodic >> lane) & 1u) y = ff_wrap_unit(y);
-          }
-          if (__all_sync(0xffffffffu, ff_in_unit(y))) {
-            x = y;
-            if (lane < D) propf[cnt][lane] = y;
-            if (lane == 0) cstep[cnt] = t + q;
-            ++cnt;
-          }
-        }
-        __syncwarp();
-        if (lane == 0) {
-          s_nin = cnt;
-          s_end = cnt == m ? cstep[m - 1] : t + W - 1;
-        }
-      }
-      __syncthreads();
-      nin = s_nin;
-    } else {
     const unsigned mask = __ballot_sync(0xffffffffu, in);
     if (lane == 0) wcount[warp] = __popc(mask);
     __syncthreads();
