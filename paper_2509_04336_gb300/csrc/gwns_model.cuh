@@ -493,14 +493,6 @@ __device__ inline void taylorf2_setup_lean(const EventDev& ev, const LeanTheta& 
   p.hh = hh;
 }
 
-// Lean constants from a physical theta (ns_likelihood_batch in the mixed paths).
-__device__ inline void theta_to_lean(const double* th, LeanTheta& t) {
-  t.mc = th[0]; t.q = th[1]; t.chi1 = th[2]; t.chi2 = th[3];
-  t.dl = (float)th[4]; t.ci = (float)cos(th[5]); t.psi = (float)th[6];
-  t.phic = th[7]; t.tc = th[8]; t.ra = th[9];
-  sincos(th[10], &t.sdec, &t.cdec);
-}
-
 // ---------------------------------------------------------------- per-bin accumulation
 struct AccF64 {
   double re[kMaxDet], im[kMaxDet];

@@ -536,20 +536,6 @@ __device__ inline void setup_from_unit(const EventDev& ev, const double* u, Walk
   }
 }
 
-template <int PREC, int WF>
-__device__ inline void setup_from_theta(const EventDev& ev, const double* th, WalkerParams& P) {
-  if (PREC == 0) {
-    double sd, cd;
-    sincos(th[10], &sd, &cd);
-    taylorf2_setup<WF>(ev, th, cos(th[5]), sd, cd, P);
-  } else {
-    LeanTheta t;
-    theta_to_lean(th, t);
-    taylorf2_setup_lean<WF>(ev, t, P);
-    if (PREC == 2) make_ff<WF>(ev, P);
-  }
-}
-
 // ---------------------------------------------------------------- likelihood batch
 // ln L of n proposals, in [n][11] physical vectors or (UNIT) [n][D] unit-cube points: one CTA takes a
 // tile of `tile` of them.  The four warps form the tile's constants together (setup_tile: a
@@ -1114,10 +1100,12 @@ __device__ __forceinline__ ff ff_wrap_unit(ff x) {
 
 // The acceptance walk of mode 2.  The round of walk_kernel, restructured so that its serial
 // part is short:
-//  1. every thread forms the move of one candidate step of the window exactly, in float-float
-//     arithmetic (the DE scale's logarithm, the survivors' float-float difference, the periodic
-//     wrap, the bounds test) -- there is no FP32 screen and no one-warp recheck -- and a ballot
-//     compacts the first m in-bounds moves;
+//  1. every thread draws one candidate step of the window and screens its move in FP32; the steps
+//     that may stay in the cube (at most 32) are moved exactly, in float-float arithmetic (the DE
+//     scale's logarithm, the survivors' float-float difference, the periodic wrap, the bounds test),
+//     candidate a lane, coordinates over the warps, and ballots compact the first m in-bounds
+//     moves (launches with flow proposals or relative binning form every step's exact move on its
+//     thread);
 //  2. the proposal constants of the round run on all four warps at once (tf2_split_first /
 //     tf2_split_second, pd_split_first / pd_split_second: independent chains, then the
 //     products; the IMRPhenomD form's continuity constants and its region boundaries and
