@@ -349,3 +349,28 @@ def test_flow_accept_weight_shortens_walks_by_its_rule():
     lz, lz_err, n_like = runs[wt]
     assert abs(lz - ref["log_z"]) < 4 * math.hypot(max(lz_err, 0.05), max(ref["log_z_err"], 0.05))
     assert n_like < runs[0.0][2]
+
+
+@pytest.mark.parametrize("n", [1, 63, 64, 65, 128, 191])
+def test_gradient_at_tile_edges(n):
+    # Tiles of 64 points: a part that begins at a tile's edge has the tile's own partial gradient, so
+    # n g(n) is the sum of the parts' up to the FP32 additions and scalings (a few roundings of
+    # 2^-24 each on sums of the parts' size: 2^-21 of the sum of their magnitudes), and points
+    # that are not there add nothing.
+    w, ev, h = flow_handle("bbh11_3det_4s_taylorf2", layers=3)
+    try:
+        D = w.n_dim
+        f, p = random_params(D, 3, 6)
+        set_both(h, f, p, D, 7)
+        u = np.random.default_rng(n).uniform(0.02, 0.98, (n, D))
+        loss, g = gwns.ns_flow_grad(h, 0, u)
+        parts = [(len(x), *gwns.ns_flow_grad(h, 0, x)) for x in (u[i:i + 64] for i in range(0, n, 64))]
+    finally:
+        gwns.ns_free(h)
+    total = sum(k * gp.astype(np.float64) for k, _, gp in parts)
+    size = sum(k * np.abs(gp.astype(np.float64)) for k, _, gp in parts)
+    assert np.all(np.abs(n * g.astype(np.float64) - total) <= 2.0 ** -21 * size)
+    assert abs(n * loss - sum(k * lp for k, lp, _ in parts)) <= 1e-12 * n * max(1.0, abs(loss))
+    if n in (1, 65):
+        ol, og = F.loss_and_grad(f, u, bf16=True)
+        assert np.all(np.abs(g.astype(np.float64) - og) <= gradient_bound(f, u, og))
