@@ -1,6 +1,7 @@
 // api.cu -- C ABI of libgwns: handle lifetime, input checks, event preprocessing and the
 // entry points that evaluate the model (ns_waveform, ns_likelihood_batch, ns_walk_batch).
 // The nested-sampling driver entry points live in nested.cu.
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -573,12 +574,12 @@ bool walk_uses_flow(const ns_handle* h, int e) {
   return E.flow.enabled && E.flow.p_flow > 0.0;
 }
 
-bool walk_extras(const ns_handle* h, int e) { return h->events[e].dev.rb_nb > 0 || walk_uses_flow(h, e); }
+int walk_extras(const ns_handle* h, int e) { return walk_uses_flow(h, e) ? 2 : h->events[e].dev.rb_nb > 0 ? 1 : 0; }
 
-bool walk_extras(const ns_handle* h) {
-  for (int e = 0; e < (int)h->events.size(); ++e)
-    if (walk_extras(h, e)) return true;
-  return false;
+int walk_extras(const ns_handle* h) {
+  int x = 0;
+  for (int e = 0; e < (int)h->events.size(); ++e) x = std::max(x, walk_extras(h, e));
+  return x;
 }
 
 cudaError_t copy_on(ns_handle* h, void* dst, const void* src, size_t bytes, cudaMemcpyKind kind) {

@@ -78,11 +78,11 @@ cudaError_t turn_table_upload(cudaStream_t s);
 // copy survf of the n_surv survivor coordinates T.surv; clears clear[0], clear[1] (if not null).
 cudaError_t launch_walk_prepare(const WalkTask& T, WalkTask* d_task, int32_t* d_blk_task, int32_t* d_blk_local,
                                 float2* d_survf, int32_t* clear, size_t n_surv, cudaStream_t s);
-// Block b walks walker blk_local[b] of task blk_task[b].  extras: some task of the launch uses
-// flow proposals or the relative-binning likelihood (false lets mode 2 run a walk kernel
-// compiled without those paths).  chain: the walks may look ahead over acceptances.
+// Block b walks walker blk_local[b] of task blk_task[b].  extras: what some task of the launch uses
+// (2 flow proposals, 1 the relative-binning likelihood only, 0 neither), which lets mode 2 run a
+// walk kernel compiled without the rest.  chain: the walks may look ahead over acceptances.
 cudaError_t launch_walk(int precision, int waveform, int n_det, const EventDev* d_evs, WalkTask* d_tasks,
                         const int32_t* d_blk_task, const int32_t* d_blk_local, int n_blocks, cudaStream_t s,
-                        bool extras, bool chain);
+                        int extras, bool chain);
 
 }  // namespace gwns

@@ -43,7 +43,7 @@ cudaError_t launch_unit_likelihood_p(int waveform, int n_det, const EventDev* d_
 template <int P>
 cudaError_t launch_walk_p(int waveform, int n_det, const EventDev* d_evs, WalkTask* d_tasks,
                           const int32_t* d_blk_task, const int32_t* d_blk_local, int n_blocks, cudaStream_t s,
-                          bool extras, bool chain);
+                          int extras, bool chain);
 template <int P>
 cudaError_t launch_hrss_p(int waveform, int n_det, const EventDev* d_evs, WalkTask* d_tasks,
                           const int32_t* d_blk_task, const int32_t* d_blk_local, int n_blocks, cudaStream_t s);
@@ -66,7 +66,7 @@ cudaError_t launch_unit_likelihood(int precision, int waveform, int n_det, const
 
 cudaError_t launch_walk(int precision, int waveform, int n_det, const EventDev* d_evs, WalkTask* d_tasks,
                         const int32_t* d_blk_task, const int32_t* d_blk_local, int n_blocks, cudaStream_t s,
-                        bool extras, bool chain) {
+                        int extras, bool chain) {
   if (n_blocks <= 0) return cudaSuccess;
   if (precision == 0)
     return launch_walk_p<0>(waveform, n_det, d_evs, d_tasks, d_blk_task, d_blk_local, n_blocks, s, extras, chain);

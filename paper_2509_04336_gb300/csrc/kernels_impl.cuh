@@ -681,14 +681,14 @@ __global__ void __launch_bounds__(kThreads) waveform_kernel(const EventDev* __re
 // A stand-alone walk has no batch before it: a fixed depth of 16 dropped 9 of 10 evaluations at
 // p = 0.6.  spec_cap 0 keeps the task's depth, over rejections: a depth fixed by the user, and the
 // sampler's walks, whose batch rule knows p (their own estimates, noisier, gained nothing).  Any choice gives the same
-// chain.  PAD4: rounds of a warp per proposal, padded to a multiple of four.  CH: compiled with the
+// chain.  pad4: rounds of a warp per proposal, padded to a multiple of four.  CH: compiled with the
 // look-ahead over acceptances.
 struct Round {
   int depth;
   bool chain;
 };
-template <bool PAD4, bool CH>
-__device__ __forceinline__ Round next_round(const WalkTask& T, int n_acc, int n_like) {
+template <bool CH>
+__device__ __forceinline__ Round next_round(const WalkTask& T, bool pad4, int n_acc, int n_like) {
   Round r;
   r.depth = T.spec < 1 ? 1 : (T.spec > kSpecMax ? kSpecMax : T.spec);
   r.chain = CH && T.spec_cap > 0 && 2 * n_acc > n_like;
@@ -697,7 +697,7 @@ __device__ __forceinline__ Round next_round(const WalkTask& T, int n_acc, int n_
     r.depth = (int)(1.4f * ((float)n_like + (float)r.depth) / ((float)ends + 1.4f) + 0.5f);
     r.depth = min(max(r.depth, 1), min(T.spec_cap, kSpecMax));
   }
-  if (PAD4) r.depth = min((r.depth + 3) & ~3, kSpecMax);
+  if (pad4) r.depth = min((r.depth + 3) & ~3, kSpecMax);
   return r;
 }
 
@@ -784,7 +784,7 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel(const EventDev* __res
   const int sw = s_setup_warp;
   const bool use_flow = !CH && T.flow != nullptr && T.p_flow > 0.0;
   const double p_flow = T.p_flow;
-  Round rd = next_round<false, CH>(T, 0, 0);
+  Round rd = next_round<CH>(T, false, 0, 0);
   if (use_flow) {
     const float lq = flow_logq_cta(*T.flow, u, fscr);
     if (threadIdx.x == 0) s_logq = lq;
@@ -1062,7 +1062,7 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel(const EventDev* __res
         if (T.status && rank == 0) atomicOr(T.status, 1);
       }
       s_next = nxt;
-      s_round = next_round<false, CH>(T, n_acc, n_like);
+      s_round = next_round<CH>(T, false, n_acc, n_like);
     }
     __syncthreads();
     t = s_next;
@@ -1104,8 +1104,7 @@ __device__ __forceinline__ ff ff_wrap_unit(ff x) {
 //     that may stay in the cube (at most 32) are moved exactly, in float-float arithmetic (the DE
 //     scale's logarithm, the survivors' float-float difference, the periodic wrap, the bounds test),
 //     candidate a lane, coordinates over the warps, and ballots compact the first m in-bounds
-//     moves (launches with flow proposals or relative binning form every step's exact move on its
-//     thread);
+//     moves (launches with flow proposals form every step's exact move on its thread);
 //  2. the proposal constants of the round run on all four warps at once (tf2_split_first /
 //     tf2_split_second, pd_split_first / pd_split_second: independent chains, then the
 //     products; the IMRPhenomD form's continuity constants and its region boundaries and
@@ -1121,14 +1120,18 @@ __device__ __forceinline__ ff ff_wrap_unit(ff x) {
 // 13.8 -> 7.1 ms (acceptance 0.4 to 0.7 a call).
 // The DE move is the walk's, u' = u + gamma (u_a - u_b), with the position and the survivors as
 // float pairs (~48 significant bits): the chain is the FP64 chain up to rounding at ~1e-14.
-// A TaylorF2 round is padded to a multiple of four proposals: its warp-per-proposal likelihood
-// phase takes as long for 1 or 5 proposals as for 4 or 8, and the padding only advances the
-// chain further.  The IMRPhenomD form (thousands of bins a proposal) runs each proposal on the
-// whole CTA instead.
-template <int NDET, int WF, bool XF, bool CH>
+// A TaylorF2 or relative-binning round is padded to a multiple of four proposals: its
+// warp-per-proposal likelihood phase takes as long for 1 or 5 proposals as for 4 or 8, and the
+// padding only advances the chain further.  The full grid of the IMRPhenomD form (thousands of bins a
+// proposal) runs each proposal on the whole CTA instead.
+// Relative binning runs without the flow paths (X 1), with the moves of step 1 and the padding: 1000
+// walkers x 240 steps, IMRPhenomD, 122 coarse bins, 7.17 -> 6.57 ms.  Its round is bound by the float-float
+// chains of a proposal's constants and moves; the likelihood of the coarse bins is short.
+template <int NDET, int WF, int X, bool CH>
 __global__ void __launch_bounds__(kThreads, 4) walk_kernel_ff(const EventDev* __restrict__ evs, WalkTask* tasks,
                                                             const int32_t* __restrict__ blk_task,
                                                             const int32_t* __restrict__ blk_local) {
+  constexpr bool XF = X == 2;   // flow proposals
   constexpr int NV = NVals<NDET, WF>::value;
   __shared__ WalkerParams P[kSpecMax];
   __shared__ ff propf[kSpecMax][kMaxDim];
@@ -1193,7 +1196,7 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel_ff(const EventDev* __
   const int sw = s_setup_warp;
   const bool use_flow = XF && T.flow != nullptr && T.p_flow > 0.0;
   const double p_flow = T.p_flow;
-  Round rd = next_round<WF == 0, CH>(T, 0, 0);
+  Round rd = next_round<CH>(T, WF == 0 || (X >= 1 && ev.rb_nb > 0), 0, 0);
   if (use_flow) {
     const float lq = flow_logq_cta(*T.flow, u, fscr);
     if (threadIdx.x == 0) s_logq = lq;
@@ -1367,7 +1370,7 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel_ff(const EventDev* __
         nin = s_nin;
       }
     } else {
-      // 1. flow proposals or relative binning: the exact move of one candidate step per thread
+      // 1. flow proposals: the exact move of one candidate step per thread
       const int W = min(min(kThreads, max(32, 4 * m)), n_steps - t);
     const int step = t + (int)threadIdx.x;
     int in = 0, isf = 0;
@@ -1494,7 +1497,7 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel_ff(const EventDev* __
     // 3. likelihoods
     constexpr int V = Pow2Vals<NV>::value;
     constexpr int group = 32 / V;
-    const bool rb = XF && ev.rb_nb > 0;
+    const bool rb = X >= 1 && ev.rb_nb > 0;
     // whole-CTA evaluations: proposals evaluated, the last accepted one and its ln L, the one that
     // ended the round's guess
     int neval = nin, pd_hit = -1, pd_end = -1;
@@ -1620,7 +1623,7 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel_ff(const EventDev* __
           if (T.status) atomicOr(T.status, 1);
         }
         s_next = nxt;
-        s_round = next_round<WF == 0, CH>(T, n_acc, n_like);
+        s_round = next_round<CH>(T, WF == 0 || (X >= 1 && ev.rb_nb > 0), n_acc, n_like);
       }
     }
     __syncthreads();
@@ -2233,35 +2236,39 @@ cudaError_t launch_unit_likelihood_p(int waveform, int n_det, const EventDev* d_
   return cudaGetLastError();
 }
 
-// Mode 2 runs the float-float walk; modes 0 and 1 the FP64-recheck walk.  A launch whose tasks use
-// neither flow proposals nor the relative-binning likelihood (extras false) runs the float-float
-// walk compiled without those paths (a smaller kernel: its round is short and instruction fetch is
-// among its first stalls).  Both properties of an event are fixed before its first ns_step
-// (ns_relbin_set is refused after it), so the sampler's captured batch graphs keep a valid choice.
+// Mode 2 runs the float-float walk; modes 0 and 1 the FP64-recheck walk.  extras: 0 no task of the
+// launch uses flow proposals or the relative-binning likelihood, 1 relative binning only, 2 flow
+// proposals -- each runs the float-float walk compiled without what it does not use (a smaller
+// kernel: its round is short and instruction fetch is among its first stalls).  Both properties of
+// an event are fixed before its first ns_step (ns_relbin_set is refused after it), so the sampler's
+// captured batch graphs keep a valid choice.
 // `chain` launches (stand-alone walks) take the kernels that can look ahead over acceptances: their
 // acceptance may be anything (500 walkers x 600 steps at 0.87 acceptances a call, 4,017 bins: 4.85 ->
 // 2.1 ms).  The sampler's walks accept a few per cent of their calls from the first batches on, and
 // there the larger kernel costs 5 % (ten batches: 17.9 -> 19.0 ms of walks), so they take the plain
-// one; so do flows, and relative binning, which gained nothing (7.2 -> 7.5 ms).
-// The float-float walk's three variants are compiled in units of their own (GWNS_FF_WALK: parallel
-// builds).
+// one; so do flows and the IMRPhenomD form with relative binning (1000 walkers x 240 steps at 0.6: 6.6
+// ms without, 7.4 ms with it; TaylorF2 with relative binning at 0.85: 2.6 -> 1.2 ms).
+// The float-float walk's variants are compiled in units of their own (GWNS_FF_WALK: parallel builds).
 #define GWNS_WALK_ARGS \
   int waveform, int n_det, const EventDev *d_evs, WalkTask *d_tasks, const int32_t *d_blk_task, \
       const int32_t *d_blk_local, int n_blocks, cudaStream_t s
-cudaError_t launch_walk_ff_plain(GWNS_WALK_ARGS);    // kernels_p2w.cu
-cudaError_t launch_walk_ff_extras(GWNS_WALK_ARGS);   // kernels_p2.cu
-cudaError_t launch_walk_ff_chain(GWNS_WALK_ARGS);    // kernels_p2c.cu
-#define GWNS_FF_WALK(NAME, XF, CH)                                                                                   \
+cudaError_t launch_walk_ff_plain(GWNS_WALK_ARGS);         // kernels_p2w.cu
+cudaError_t launch_walk_ff_chain(GWNS_WALK_ARGS);         // kernels_p2c.cu
+cudaError_t launch_walk_ff_relbin(GWNS_WALK_ARGS);        // kernels_p2r.cu
+cudaError_t launch_walk_ff_relbin_chain(GWNS_WALK_ARGS);  // kernels_p2r.cu, TaylorF2
+cudaError_t launch_walk_ff_flow(GWNS_WALK_ARGS);          // kernels_p2.cu
+#define GWNS_FF_WALK(NAME, X, CH)                                                                                    \
   cudaError_t NAME(GWNS_WALK_ARGS) {                                                                                 \
-    GWNS_DISPATCH_W(GWNS_FF_WALK_ONE_##XF##CH, 2)                                                                    \
+    GWNS_DISPATCH_W(GWNS_FF_WALK_ONE_##X##CH, 2)                                                                     \
     return cudaGetLastError();                                                                                       \
   }
-#define GWNS_FF_WALK_ONE_00(P_, N, W) \
-  walk_kernel_ff<N, W, false, false><<<n_blocks, kThreads, 0, s>>>(d_evs, d_tasks, d_blk_task, d_blk_local)
-#define GWNS_FF_WALK_ONE_10(P_, N, W) \
-  walk_kernel_ff<N, W, true, false><<<n_blocks, kThreads, 0, s>>>(d_evs, d_tasks, d_blk_task, d_blk_local)
-#define GWNS_FF_WALK_ONE_01(P_, N, W) \
-  walk_kernel_ff<N, W, false, true><<<n_blocks, kThreads, 0, s>>>(d_evs, d_tasks, d_blk_task, d_blk_local)
+#define GWNS_FF_WALK_RUN(N, W, X, CH) \
+  walk_kernel_ff<N, W, X, CH><<<n_blocks, kThreads, 0, s>>>(d_evs, d_tasks, d_blk_task, d_blk_local)
+#define GWNS_FF_WALK_ONE_00(P_, N, W) GWNS_FF_WALK_RUN(N, W, 0, false)
+#define GWNS_FF_WALK_ONE_01(P_, N, W) GWNS_FF_WALK_RUN(N, W, 0, true)
+#define GWNS_FF_WALK_ONE_10(P_, N, W) GWNS_FF_WALK_RUN(N, W, 1, false)
+#define GWNS_FF_WALK_ONE_11(P_, N, W) GWNS_FF_WALK_RUN(N, W, 1, true)
+#define GWNS_FF_WALK_ONE_20(P_, N, W) GWNS_FF_WALK_RUN(N, W, 2, false)
 
 // Modes 0 and 1 are bound by the FP64 pipe of a walker's SM (half of a round of eight proposals),
 // so a launch of few walkers spreads each over a cluster of CTAs: every rank runs the moves, the
@@ -2288,9 +2295,11 @@ void launch_walk_f64(bool chain, int ranks, int n_blocks, cudaStream_t s, const 
 template <int P>
 cudaError_t launch_walk_p(int waveform, int n_det, const EventDev* d_evs, WalkTask* d_tasks,
                           const int32_t* d_blk_task, const int32_t* d_blk_local, int n_blocks, cudaStream_t s,
-                          bool extras, bool chain) {
+                          int extras, bool chain) {
   if constexpr (P == 2) {
-    const auto f = extras ? launch_walk_ff_extras : chain ? launch_walk_ff_chain : launch_walk_ff_plain;
+    const auto f = extras == 2 ? launch_walk_ff_flow
+                               : extras == 1 ? (chain && waveform == 0 ? launch_walk_ff_relbin_chain : launch_walk_ff_relbin)
+                                             : (chain ? launch_walk_ff_chain : launch_walk_ff_plain);
     return f(waveform, n_det, d_evs, d_tasks, d_blk_task, d_blk_local, n_blocks, s);
   } else {
     // the largest of 4, 2 and 1 ranks that gives every CTA an SM of its own (50 walkers of 1,969 bins,
@@ -2299,9 +2308,9 @@ cudaError_t launch_walk_p(int waveform, int n_det, const EventDev* d_evs, WalkTa
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    const int ranks = extras ? 1 : 4 * n_blocks <= sms ? 4 : 2 * n_blocks <= sms ? 2 : 1;
+    const int ranks = extras == 2 ? 1 : 4 * n_blocks <= sms ? 4 : 2 * n_blocks <= sms ? 2 : 1;
 #define GWNS_WALK(P_, N, W) \
-  launch_walk_f64<P_, N, W>(chain && !extras, ranks, n_blocks, s, d_evs, d_tasks, d_blk_task, d_blk_local)
+  launch_walk_f64<P_, N, W>(chain && extras != 2, ranks, n_blocks, s, d_evs, d_tasks, d_blk_task, d_blk_local)
     GWNS_DISPATCH_W(GWNS_WALK, P)
 #undef GWNS_WALK
     return cudaGetLastError();

@@ -10,7 +10,7 @@ template cudaError_t launch_likelihood_p<0>(int, int, const EventDev*, const dou
 template cudaError_t launch_unit_likelihood_p<0>(int, int, const EventDev*, const double*, int, double*,
                                                   cudaStream_t);
 template cudaError_t launch_walk_p<0>(int, int, const EventDev*, WalkTask*, const int32_t*, const int32_t*, int,
-                                       cudaStream_t, bool, bool);
+                                       cudaStream_t, int, bool);
 template cudaError_t launch_hrss_p<0>(int, int, const EventDev*, WalkTask*, const int32_t*, const int32_t*, int,
                                        cudaStream_t);
 
