@@ -780,7 +780,9 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel(const EventDev* __res
   const uint64_t t0 = threadIdx.x == 0 ? global_ns() : 0ull;
   const double de_scale = 2.38 / sqrt(2.0 * (double)D);
   const float de_scale32 = (float)de_scale;
-  __syncthreads();
+  // a rank stores into the other ranks' shared memory in its first round: not before they run
+  if (CL) cluster.sync();
+  else __syncthreads();
   const int sw = s_setup_warp;
   const bool use_flow = !CH && T.flow != nullptr && T.p_flow > 0.0;
   const double p_flow = T.p_flow;

@@ -52,3 +52,31 @@ def test_chain_does_not_depend_on_the_launch(precision, name, f_max, depth):
             assert np.array_equal(a, b[:20])
     finally:
         gwns.ns_free(h)
+
+
+@pytest.mark.parametrize("precision", [synth.PREC_FP64, synth.PREC_MIXED])
+def test_walks_of_one_round(precision):
+    # one or two steps: a walk's first round is its last, so what the ranks exchange in it is all
+    w, ev = event("four_param_2det_taylorf2", f_max=60.0)
+    u, th = prior_draws(w, ev, 90, 8)
+    h = gwns.ns_init([gwns.make_config(w, priors(w, ev), precision=precision, spec_depth=8)], [ev])
+    try:
+        lnl = np.zeros(90)
+        gwns.ns_likelihood_batch(h, 0, th, lnl)
+        star = float(np.quantile(lnl, 0.1))
+        above = np.where(lnl > star)[0]
+        pick = above[np.arange(160) % len(above)]
+        for steps in (1, 2):
+            def walk(n):
+                out = [np.zeros((n, w.n_dim)), np.zeros(n), np.zeros(n, np.int32), np.zeros(n, np.int32)]
+                gwns.ns_walk_batch(h, 0, np.ascontiguousarray(u), np.ascontiguousarray(u[pick[:n]]),
+                                   np.ascontiguousarray(lnl[pick[:n]]), star, steps, 1, 0, *out)
+                return out
+
+            full = walk(160)
+            assert full[3].sum() > 0
+            for n in (1, 38, 76):
+                for a, b in zip(walk(n), full):
+                    assert np.array_equal(a, b[:n]), n
+    finally:
+        gwns.ns_free(h)
