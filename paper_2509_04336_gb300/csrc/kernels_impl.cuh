@@ -15,6 +15,7 @@
 
 #include "flow.cuh"
 #include "gwns_internal.h"
+#include "screen.h"
 #include "setup_split.cuh"
 
 namespace gwns {
@@ -29,12 +30,10 @@ __device__ unsigned int g_walk_sm_arrivals[256];
 constexpr int kWarps = kThreads / 32;
 constexpr int kMaxVals = 3 * kMaxDet;   // (re, im, hh) per detector
 
-// (x >> 12) + 1/2 as a float (relative error ~1e-7) from two 32-bit conversions: a 64-bit
-// integer conversion runs on the FP64 pipe.
-__device__ __forceinline__ float top52_half_f(uint64_t x) {
-  const uint64_t v = x >> 12;
-  return fmaf(__uint2float_rn((uint32_t)(v >> 20)), 1048576.0f, __uint2float_rn((uint32_t)(v & 0xFFFFFull)) + 0.5f);
-}
+// the hardware base-2 logarithm, for the screens of DE steps (screen.h)
+struct FastLog2 {
+  __device__ __forceinline__ float operator()(float x) const { return __log2f(x); }
+};
 
 __device__ __forceinline__ uint64_t global_ns() {
   uint64_t t;
@@ -865,15 +864,9 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel(const EventDev* __res
       float sc = 1.0f;
       if ((A.v[2] >> 63) == 0ull) {
         Philox4 B = philox4x64((uint64_t)step, wid, it, 1ull, T.key0, T.key1);
-        // log2 U_i = log2((x_i >> 12) + 1/2) - 52, each factor's integer rounded to float
-        // (relative error ~1e-7, no truncation, no underflow of the product)
-        float l2 = __log2f(top52_half_f(B.v[0])) + __log2f(top52_half_f(B.v[1])) + __log2f(top52_half_f(B.v[2])) +
-                   __log2f(top52_half_f(B.v[3])) - 208.0f;
-        sc = de_scale32 * (-0.25f * 0.6931471805599453f * l2);
+        sc = screen_scale(B.v, de_scale32, FastLog2{});
       }
-      // |x32 - x64| stays below ~1e-7 (1 + |s|) plus the log2 error times |s|: a margin of
-      // 1e-5 (1 + |s|) never rejects a step that the exact FP64 test accepts
-      const float margin = 1e-5f * (1.0f + fabsf(sc));
+      const float margin = screen_margin(sc);
       maybe = 1;
       if (T.survf) {
         const float2* ua = T.survf + a * D;
@@ -1211,7 +1204,7 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel_ff(const EventDev* __
     int nin;
     if constexpr (!XF) {
       // 1a. one step a thread: its draws and, looking ahead over rejections, a FP32 screen of its move
-      //     (as in walk_kernel: the margin never rejects a step that the exact test accepts).  Four
+      //     (as in walk_kernel; the margin never rejects a step that the exact test accepts: screen.h).  Four
       //     moves of five leave the cube, and the exact move of one is ~700 float-float
       //     instructions: it is formed for the steps that may stay only.  Looking ahead over
       //     acceptances: the next 32 steps, unscreened.
@@ -1249,11 +1242,9 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel_ff(const EventDev* __
           }
           float sc = 1.0f;
           if (draw_scale) {
-            const float l2 = __log2f(top52_half_f(B.v[0])) + __log2f(top52_half_f(B.v[1])) +
-                             __log2f(top52_half_f(B.v[2])) + __log2f(top52_half_f(B.v[3])) - 208.0f;
-            sc = de_scale.h * (-0.25f * 0.6931471805599453f * l2);
+            sc = screen_scale(B.v, de_scale.h, FastLog2{});
           }
-          const float margin = 1e-5f * (1.0f + fabsf(sc));
+          const float margin = screen_margin(sc);
 #pragma unroll
           for (int d = 0; d < kMaxDim; ++d) {
             const float x = uf[d < D ? d : D - 1].h + sc * (va[d] - vb[d]);
