@@ -1099,7 +1099,12 @@ __device__ __forceinline__ ff ff_wrap_unit(ff x) {
 //     that may stay in the cube (at most 32) are moved exactly, in float-float arithmetic (the DE
 //     scale's logarithm, the survivors' float-float difference, the periodic wrap, the bounds test),
 //     candidate a lane, coordinates over the warps, and ballots compact the first m in-bounds
-//     moves (launches with flow proposals form every step's exact move on its thread);
+//     moves.  Launches with flow proposals, and the sampler's own TaylorF2 walks, form every step's
+//     exact move on its thread instead: the sampler's long windows fill the threads, and the
+//     screen's draws, compaction and second pass cost more than the exact moves they save (walks
+//     of a 4-parameter run to ln Z 15.4 ms screened, 14.6 not; of an 11-parameter one 160.7 and 159.3,
+//     6 late batches of it on relative binning 27.1 and 26.5; but 8 batches of the 16,225-bin
+//     IMRPhenomD form 354 and 385: its walks screen);
 //  2. the proposal constants of the round run on all four warps at once (tf2_split_first /
 //     tf2_split_second, pd_split_first / pd_split_second: independent chains, then the
 //     products; the IMRPhenomD form's continuity constants and its region boundaries and
@@ -1127,6 +1132,7 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel_ff(const EventDev* __
                                                             const int32_t* __restrict__ blk_task,
                                                             const int32_t* __restrict__ blk_local) {
   constexpr bool XF = X == 2;   // flow proposals
+  constexpr bool kScreen = !XF && (CH || WF == 1);   // step 1: screened moves
   constexpr int NV = NVals<NDET, WF>::value;
   __shared__ WalkerParams P[kSpecMax];
   __shared__ ff propf[kSpecMax][kMaxDim];
@@ -1148,8 +1154,8 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel_ff(const EventDev* __
   __shared__ int wcount[kWarps];
   __shared__ unsigned wmask[kWarps];
   // candidates of a round: the step (complemented: unit scale), its survivors, the scale's uniforms
-  __shared__ int cand_step[XF ? 1 : 32], cand_a[XF ? 1 : 32], cand_b[XF ? 1 : 32];
-  __shared__ uint64_t cand_u[XF ? 1 : 32][4];
+  __shared__ int cand_step[kScreen ? 32 : 1], cand_a[kScreen ? 32 : 1], cand_b[kScreen ? 32 : 1];
+  __shared__ uint64_t cand_u[kScreen ? 32 : 1][4];
   __shared__ int s_next, s_setup_warp, s_end, s_needq, s_nin;
   __shared__ Round s_round;
   __shared__ int s_isflow[kSpecMax];
@@ -1202,7 +1208,7 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel_ff(const EventDev* __
     const int abort_flag = threadIdx.x == 0 ? walk_abort_flag(T) : 0;
     const int m = rd.depth;
     int nin;
-    if constexpr (!XF) {
+    if constexpr (kScreen) {
       // 1a. one step a thread: its draws and, looking ahead over rejections, a FP32 screen of its move
       //     (as in walk_kernel; the margin never rejects a step that the exact test accepts: screen.h).  Four
       //     moves of five leave the cube, and the exact move of one is ~700 float-float
@@ -1363,7 +1369,7 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel_ff(const EventDev* __
         nin = s_nin;
       }
     } else {
-      // 1. flow proposals: the exact move of one candidate step per thread
+      // 1. the exact move of one candidate step per thread (or its flow proposal)
       const int W = min(min(kThreads, max(32, 4 * m)), n_steps - t);
     const int step = t + (int)threadIdx.x;
     int in = 0, isf = 0;
