@@ -719,12 +719,14 @@ extern "C" int ns_step(ns_handle* h, int max_batches, ns_progress* progress) {
     // active bins (with relative binning: edges plus exact-range bins) is a short likelihood whose
     // rounds are dominated by fixed costs (largest cap); a longer one costs a full evaluation per
     // speculative proposal (small cap) -- except in the float-float IMRPhenomD-form walk, whose
-    // rounds end at their first acceptance and evaluate nothing in vain (largest cap).
+    // rounds end at their first acceptance and evaluate nothing in vain (largest cap); not so on
+    // relative binning, which evaluates a round's proposals side by side, a warp each.
     if (h->tune && !h->tune_guessed && it_now >= 1) {
       double bins = 0.0, evals = 0.0;
+      bool early_end = h->precision == NS_PREC_MIXED_FF && h->waveform == NS_WAVEFORM_PHENOMD_FORM;
       for (auto& S : h->host_ns) { bins += (double)S.n_bins_eval; evals += (double)S.n_spec_eval; }
-      const bool short_lik = (evals > 0.0 && bins < 1024.0 * evals) ||
-                             (h->precision == NS_PREC_MIXED_FF && h->waveform == NS_WAVEFORM_PHENOMD_FORM);
+      for (auto& E : h->events) early_end = early_end && E.dev.rb_nb == 0;
+      const bool short_lik = (evals > 0.0 && bins < 1024.0 * evals) || early_end;
       const int cap = h->precision == 0 ? (short_lik ? 8 : 2) : (short_lik ? 32 : 4);
       if ((r = set_spec_cap(h, cap))) return r;
       h->tune_best = cap;
