@@ -156,20 +156,6 @@ __device__ __forceinline__ void ff_extrinsic(const EventDev& ev, const ff* x, FF
   ff_prior_dec(ev, x, c.sd, c.cd);
 }
 
-// Prior transform, masses and the 3.5PN coefficients from the float-float unit-cube point x
-// (requires ev.ff_setup).
-__device__ inline void ff_core(const EventDev& ev, const ff* x, FFCore& c) {
-  ff_extrinsic(ev, x, c);
-  c.q = ff_prior_lin(ev, 1, x);
-  c.chi1 = ff_prior_lin(ev, 2, x);
-  c.chi2 = ff_prior_lin(ev, 3, x);
-  c.phic = ff_prior_lin(ev, 7, x);
-  ff_mass_ratio(c);
-  ff_mass_scales(c);
-  ff_pn_coeffs(c);
-  ff_log_and_prefactor(c);
-}
-
 // The products that make the TaylorF2 basis coefficients (cycles): C_j for j in [j0, j1).
 __device__ inline void ff_tf2_coeff_range(const FFCore& c, int j0, int j1, WalkerParams& p) {
   const ff pre = c.pre, c1 = c.c1;
@@ -199,11 +185,6 @@ __device__ inline void ff_tf2_phase0(const FFCore& c, WalkerParams& p) {
   ph0 = ff_add_f(ph0, -0.125f);
   p.ph0h = ph0.h;
   p.ph0l = ph0.l;
-}
-// TaylorF2 phase coefficients on the basis and the phase constant, float-float.
-__device__ inline void ff_tf2_coeffs(const FFCore& c, WalkerParams& p) {
-  ff_tf2_coeff_range(c, 0, kBasis, p);
-  ff_tf2_phase0(c, p);
 }
 
 // Number of bins with f_k <= f_cut (le) or f_k < f_cut (strict), float-float comparisons.
@@ -272,20 +253,10 @@ __device__ __forceinline__ int ff_tf2_kend(const EventDev& ev, const FFCore& c) 
   return ff_bins_below(ev, ff_mul(GWNS_FF(1.0 / kSix15), c.ci3), false);
 }
 
-// Mode-2 TaylorF2 proposal constants straight from the float-float unit-cube point x.
-__device__ inline void taylorf2_setup_ff(const EventDev& ev, const ff* x, WalkerParams& p) {
-  FFCore c;
-  ff_core(ev, x, c);
-  p.k_end = ff_tf2_kend(ev, c);
-  ff_tf2_coeffs(c, p);
-  ff_projection(ev, c, p);
-  ff_tf2_hh(ev, p);
-}
-
-// The same constants formed by the warps of a CTA at once: each warp runs one part for every
-// proposal of a round (lane i: proposal i), the parts exchange through shared memory, then a
-// second pass forms the products.  The arithmetic is the one-lane setup's, split at its
-// independent chains -- first pass: (0) mass scales, ln(pi M), prefactor; (1) PN coefficients;
+// Mode-2 TaylorF2 proposal constants straight from the float-float unit-cube point x, formed by the
+// warps of a CTA at once: each warp runs one part for every proposal of a round (lane i: proposal
+// i), the parts exchange through shared memory, then a second pass forms the products.  The parts
+// are the independent chains of the setup -- first pass: (0) mass scales, ln(pi M), prefactor; (1) PN coefficients;
 // (2) sky, antenna patterns, delays; second pass: (0, 1) the basis coefficients, (2) the phase
 // constant, (3) the ISCO bin and <h|h>.  TF2Part carries (0) and (1) to the second pass.
 struct TF2Part {
@@ -340,8 +311,7 @@ __device__ inline void tf2_split_second(int part, const EventDev& ev, const TF2P
 // float-float comparisons, the ringdown frequency, damping and amplitude shape in FP32 (the
 // FP64 path's FAST variant rounds the same quantities to FP32).  Two halves that depend on the
 // TaylorF2 core only: pd_chain (continuity constants, region coefficients, phase constants) and
-// pd_bins_amp (region boundaries, amplitude shape); the one-lane setup runs both, the split setup
-// runs them on different warps.
+// pd_bins_amp (region boundaries, amplitude shape), which run on different warps.
 // Quantities both halves need: mass scales of the ringdown model and the ringdown frequency and
 // damping (units of 1/M, FP32).
 struct PDPro {
@@ -478,20 +448,10 @@ __device__ inline void pd_bins_amp(const EventDev& ev, const FFCore& c, WalkerPa
   p.hh_f = 0.0f;   // the IMRPhenomD form sums its template power per bin
 }
 
-__device__ inline void phenomd_setup_ff(const EventDev& ev, const ff* x, WalkerParams& p) {
-  FFCore c;
-  ff_core(ev, x, c);
-  ff_tf2_coeffs(c, p);
-  pd_chain(c, p);
-  pd_bins_amp(ev, c, p);
-  ff_projection(ev, c, p);
-}
-
 // The IMRPhenomD-form constants formed by the warps of a CTA at once, as tf2_split_first /
 // tf2_split_second: first pass (0) mass scales, ln(pi M), prefactor, mass ratio; (1) PN
 // coefficients and spin combinations; (2) sky, antenna patterns, delays; second pass (0, 1) the
-// TaylorF2 basis coefficients, (2) the phase constant and pd_chain, (3) pd_bins_amp.  The
-// arithmetic of every quantity is the one-lane setup's.
+// TaylorF2 basis coefficients, (2) the phase constant and pd_chain, (3) pd_bins_amp.
 struct PDPart {
   TF2Part t;
   ff q, eta, delta, chis, chia, chi1, chi2;

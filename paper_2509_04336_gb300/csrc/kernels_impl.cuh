@@ -513,20 +513,15 @@ __device__ inline bool theta_ok(const double* th) {
   return th[0] > 0.0 && th[1] > 0.0 && th[4] > 0.0;
 }
 
-// Per-walker constants of one proposal: the FP64 path uses the plain FP64 setup, the mixed
-// paths the lean one (FP64 only where the phase needs it).
+// Per-walker constants of one proposal, on one thread: the FP64 path uses the plain FP64 setup, the
+// mixed paths the lean one (FP64 only where the phase needs it; in mode 2 for priors that the
+// float-float setup of ff_setup.cuh does not transform).
 template <int PREC, int WF>
 __device__ inline void setup_from_unit(const EventDev& ev, const double* u, WalkerParams& P) {
   if (PREC == 0) {
     double th[kParams], ci, sd, cd;
     unit_to_theta(ev, u, th, &ci, &sd, &cd);
     taylorf2_setup<WF>(ev, th, ci, sd, cd, P);
-  } else if (PREC == 2 && ev.ff_setup) {
-    ff x[kMaxDim];
-#pragma unroll
-    for (int d = 0; d < kMaxDim; ++d) x[d] = d < ev.n_dim ? ff_from_double(u[d]) : ff_make(0.0f);
-    if (WF == 0) taylorf2_setup_ff(ev, x, P);
-    else phenomd_setup_ff(ev, x, P);
   } else {
     LeanTheta t;
     unit_to_lean(ev, u, t);
@@ -1492,15 +1487,10 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel_ff(const EventDev* __
           else pd_split_second(warp, ev, parts[lane], P[lane]);
         }
       } else if (warp == sw && lane < nin) {
-        if (ev.ff_setup) {
-          if (WF == 0) taylorf2_setup_ff(ev, propf[lane], P[lane]);
-          else phenomd_setup_ff(ev, propf[lane], P[lane]);
-        } else {
-          double pd[kMaxDim];
+        double pd[kMaxDim];
 #pragma unroll
-          for (int d = 0; d < kMaxDim; ++d) pd[d] = d < D ? (double)propf[lane][d].h + (double)propf[lane][d].l : 0.0;
-          setup_from_unit<2, WF>(ev, pd, P[lane]);
-        }
+        for (int d = 0; d < kMaxDim; ++d) pd[d] = d < D ? (double)propf[lane][d].h + (double)propf[lane][d].l : 0.0;
+        setup_from_unit<2, WF>(ev, pd, P[lane]);
       }
       __syncthreads();
     }
@@ -2038,15 +2028,10 @@ __global__ void __launch_bounds__(kThreads, 4) hrss_kernel_ff(const EventDev* __
           else pd_split_second(warp, ev, parts[lane], P[lane]);
         }
       } else if (warp == sw && lane < nin) {
-        if (ev.ff_setup) {
-          if (WF == 0) taylorf2_setup_ff(ev, propf[lane], P[lane]);
-          else phenomd_setup_ff(ev, propf[lane], P[lane]);
-        } else {
-          double pd[kMaxDim];
+        double pd[kMaxDim];
 #pragma unroll
-          for (int d = 0; d < kMaxDim; ++d) pd[d] = d < D ? (double)propf[lane][d].h + (double)propf[lane][d].l : 0.0;
-          setup_from_unit<2, WF>(ev, pd, P[lane]);
-        }
+        for (int d = 0; d < kMaxDim; ++d) pd[d] = d < D ? (double)propf[lane][d].h + (double)propf[lane][d].l : 0.0;
+        setup_from_unit<2, WF>(ev, pd, P[lane]);
       }
       __syncthreads();
     }
