@@ -2,16 +2,18 @@
 // forward map (log q), the inverse map (proposal tables), the maximum-likelihood gradient,
 // Adam with the bf16 weight-image update, standardisation and initialisation.
 //
-// Work layout.  A tile is 128 points; thread t of the 128-thread CTA owns point t of the
-// tile (its row of every activation and of every TMEM accumulator).  One coupling layer is
+// Work layout.  The apply kernels take tiles of 128 points; thread t of the 128-thread CTA owns
+// point t of the tile (its row of every activation and of every TMEM accumulator).  The gradient
+// kernel takes tiles of 64 points (rows 0 .. 63, the others masked) on 512 threads, four groups
+// that share the columns of the hidden layers' epilogues.  One coupling layer is
 // three products with bf16 operands staged in shared memory and FP32 accumulators in TMEM:
 //     G1 [128 x 128] = a  [128 x 16]  * W1^T      (K = 16,  one MMA)
 //     G2 [128 x 128] = h1 [128 x 128] * W2^T      (K = 128, eight MMAs)
 //     G3 [128 x 32]  = h2 [128 x 128] * W3^T      (K = 128, eight MMAs)
 // issued by thread 0 (tcgen05.mma, kind::f16), completed through tcgen05.commit on an
 // mbarrier, and read back with tcgen05.ld for the FP32 epilogues (bias, tanh, coupling).
-// Weights arrive by one bulk copy (cp.async.bulk) per layer, double-buffered in the apply
-// kernel so the next layer's copy overlaps this layer's work.
+// Weights arrive by one bulk copy (cp.async.bulk) per layer and pass, double-buffered so that the
+// next layer's copy overlaps this layer's work.
 //
 // The gradient kernel keeps each layer's inputs and activations on the way forward (40 KB a tile and
 // layer, written and read by the same CTA) and forms, per tile,

@@ -1,5 +1,6 @@
 // kernels_impl.cuh -- likelihood, waveform and acceptance-walk kernels (sm_103a).
-// Included by kernels_p{0,1,2}.cu, one translation unit per precision (parallel builds).
+// Included by the kernels_p*.cu units: one per precision (p0, p1, p2) and one per variant of the
+// float-float walk (p2w, p2c, p2r; the flow variant is in p2), for parallel builds.
 //
 // Template parameters of every kernel: PREC (0 FP64, 1 mixed with FP64 phase, 2 mixed with
 // float-float phase), NDET (detectors, 1..4) and WF (0 TaylorF2, 1 IMRPhenomD form).
@@ -366,7 +367,7 @@ __device__ __forceinline__ float tf2_ff_r0(const EventDev& ev, const WalkerParam
 }
 
 // The float-float IMRPhenomD-form phase [cycles] and amplitude shape at grid bin k, as the first
-// half of pd_accumulate_ff computes them.
+// half of pd_segment_ff computes them.
 __device__ __forceinline__ void pd_ff_r0_amp(const EventDev& ev, const WalkerParams& p, const PhenomExtra& e,
                                              int k, float& r0, float& amp) {
   const float2* g = ev.basis_ff + k;
@@ -713,14 +714,16 @@ __device__ __forceinline__ Round next_round(const WalkTask& T, bool pad4, int le
 //     tag), not on the chain, so every thread screens one candidate step in FP32 from the
 //     current position; the candidates that may lie in the cube are compacted into one warp,
 //     which redoes their draws and proposals exactly in FP64 and compacts the in-bounds ones,
-//     in step order, into at most m = task.spec slots;
+//     in step order, into at most m slots, m the round's depth (next_round).  A round that looks
+//     ahead over acceptances instead chains its moves exactly, each in-bounds one from the last;
 //  2. the four warps form the per-proposal constants together (independent chains on different
-//     warps, a proposal a lane), and the CTA evaluates the slots' likelihoods, one warp per proposal (the whole CTA per
-//     proposal when there are fewer than kWarps of them);
+//     warps, a proposal a lane), and the CTA evaluates the slots' likelihoods, one warp per
+//     proposal (the whole CTA per proposal when there are fewer than kWarps of them);
 //  3. thread 0 replays the steps in order: out-of-bounds steps reject without a likelihood
-//     call, the first in-bounds proposal with ln L > ln L* is taken and ends the round.
-//     Candidates after it were built from a position the chain has left and are redrawn
-//     from the new one in the next round.
+//     call, an in-bounds proposal with ln L > ln L* is taken, and the round ends where its guess
+//     first fails: at its first acceptance, or, looking ahead over acceptances, its first rejection.
+//     Candidates after it were built from a position the chain does not take and are redrawn
+//     from the right one in the next round.
 // The chain, the accepted and likelihood-call counts and every ln L are those of the walk
 // that takes one step at a time.  The setup warp rotates over the CTAs of an SM (an arrival
 // counter), so their FP64 work lands on different sub-partitions.
@@ -849,140 +852,141 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel(const EventDev* __res
         }
       }
     } else {
-    const int W = min(min(kThreads, max(32, 4 * m)), n_steps - t);
-    // 1a. every thread screens one candidate step in FP32
-    int maybe = 0;
-    const int step = t + (int)threadIdx.x;
-    bool fl = false;
-    if (use_flow && (int)threadIdx.x < W) {
-      Philox4 C = philox4x64((uint64_t)step, wid, it, 6ull, T.key0, T.key1);
-      if (rand_open_unit(C.v[0]) < p_flow) {
-        fl = true;
-        const float lqf = (float)T.flq[(size_t)j * T.f_stride + step];
-        maybe = logf((float)rand_open_unit(C.v[1])) < s_logq - lqf;
-      }
-    }
-    if ((int)threadIdx.x < W && !fl) {
-      Philox4 A = philox4x64((uint64_t)step, wid, it, 0ull, T.key0, T.key1);
-      uint64_t a = rand_index(A.v[0], n_s);
-      uint64_t b = rand_index(A.v[1], n_s - 1);
-      b += (b >= a) ? 1ull : 0ull;
-      float sc = 1.0f;
-      if ((A.v[2] >> 63) == 0ull) {
-        Philox4 B = philox4x64((uint64_t)step, wid, it, 1ull, T.key0, T.key1);
-        sc = screen_scale(B.v, de_scale32, FastLog2{});
-      }
-      const float margin = screen_margin(sc);
-      maybe = 1;
-      if (T.survf) {
-        const float2* ua = T.survf + a * D;
-        const float2* ub = T.survf + b * D;
-#pragma unroll
-        for (int d = 0; d < kMaxDim; ++d) {
-          if (d < D && !ev.prior[ev.dim_param[d]].periodic) {
-            float x = u32[d] + sc * (ua[d].x - ub[d].x);
-            if (!(x >= -margin && x <= 1.0f + margin)) maybe = 0;
-          }
-        }
-      } else {
-        const double* ua = T.surv + a * D;
-        const double* ub = T.surv + b * D;
-#pragma unroll
-        for (int d = 0; d < kMaxDim; ++d) {
-          if (d < D && !ev.prior[ev.dim_param[d]].periodic) {
-            float x = u32[d] + sc * ((float)ua[d] - (float)ub[d]);
-            if (!(x >= -margin && x <= 1.0f + margin)) maybe = 0;
-          }
-        }
-      }
-    }
-    unsigned mask = __ballot_sync(0xffffffffu, maybe);
-    if (lane == 0) wcount[warp] = __popc(mask);
-    __syncthreads();
-    int before = 0, total = 0;
-#pragma unroll
-    for (int w2 = 0; w2 < kWarps; ++w2) {
-      int cw = wcount[w2];
-      before += (w2 < warp) ? cw : 0;
-      total += cw;
-    }
-    const int mslot = before + __popc(mask & ((1u << lane) - 1u));
-    if (maybe && mslot < 32) mstep[mslot] = step;
-    const int nmaybe = min(total, 32);
-    __syncthreads();
-    // 1b. the setup warp redoes the maybe-in-bounds steps exactly (FP64, as the walk is
-    //     defined) and compacts the in-bounds ones into at most m slots
-    if (warp == sw) {
-      int in = 0, isf = 0;
-      float lqf = 0.0f;
-      double pr[kMaxDim];
-      const int st = lane < nmaybe ? mstep[lane] : 0;
-      if (use_flow && lane < nmaybe) {
-        Philox4 C = philox4x64((uint64_t)st, wid, it, 6ull, T.key0, T.key1);
+      const int W = min(min(kThreads, max(32, 4 * m)), n_steps - t);
+      // 1a. every thread screens one candidate step in FP32
+      int maybe = 0;
+      const int step = t + (int)threadIdx.x;
+      bool fl = false;
+      if (use_flow && (int)threadIdx.x < W) {
+        Philox4 C = philox4x64((uint64_t)step, wid, it, 6ull, T.key0, T.key1);
         if (rand_open_unit(C.v[0]) < p_flow) {
-          isf = 1;
-          lqf = (float)T.flq[(size_t)j * T.f_stride + st];
-          in = logf((float)rand_open_unit(C.v[1])) < s_logq - lqf;
-          const double* fu = T.fu + ((size_t)j * T.f_stride + st) * D;
-#pragma unroll
-          for (int d = 0; d < kMaxDim; ++d)
-            if (d < D) pr[d] = fu[d];
+          fl = true;
+          const float lqf = (float)T.flq[(size_t)j * T.f_stride + step];
+          maybe = logf((float)rand_open_unit(C.v[1])) < s_logq - lqf;
         }
       }
-      if (lane < nmaybe && !isf) {
-        Philox4 A = philox4x64((uint64_t)st, wid, it, 0ull, T.key0, T.key1);
+      if ((int)threadIdx.x < W && !fl) {
+        Philox4 A = philox4x64((uint64_t)step, wid, it, 0ull, T.key0, T.key1);
         uint64_t a = rand_index(A.v[0], n_s);
         uint64_t b = rand_index(A.v[1], n_s - 1);
         b += (b >= a) ? 1ull : 0ull;
-        double sc;
-        if ((A.v[2] >> 63) == 1ull) {
-          sc = 1.0;
-        } else {
-          Philox4 B = philox4x64((uint64_t)st, wid, it, 1ull, T.key0, T.key1);
-          double prod = __dmul_rn(__dmul_rn(__dmul_rn(rand_open_unit(B.v[0]), rand_open_unit(B.v[1])),
-                                            rand_open_unit(B.v[2])), rand_open_unit(B.v[3]));
-          sc = __dmul_rn(de_scale, __dmul_rn(-0.25, log(prod)));
+        float sc = 1.0f;
+        if ((A.v[2] >> 63) == 0ull) {
+          Philox4 B = philox4x64((uint64_t)step, wid, it, 1ull, T.key0, T.key1);
+          sc = screen_scale(B.v, de_scale32, FastLog2{});
         }
-        const double* ua = T.surv + a * D;
-        const double* ub = T.surv + b * D;
-        in = 1;
+        const float margin = screen_margin(sc);
+        maybe = 1;
+        if (T.survf) {
+          const float2* ua = T.survf + a * D;
+          const float2* ub = T.survf + b * D;
 #pragma unroll
-        for (int d = 0; d < kMaxDim; ++d) {
-          if (d < D) {
-            double x = __dadd_rn(u[d], __dmul_rn(sc, __dsub_rn(ua[d], ub[d])));
-            if (ev.prior[ev.dim_param[d]].periodic) x = __dsub_rn(x, floor(x));
-            // 0 <= x <= 1 on the bit pattern (integer pipe): +0 .. 1.0 are the patterns up
-            // to 0x3FF0000000000000; negative values and NaN compare above.  x is never -0.
-            if ((unsigned long long)__double_as_longlong(x) > 0x3FF0000000000000ull) in = 0;
-            pr[d] = x;
+          for (int d = 0; d < kMaxDim; ++d) {
+            if (d < D && !ev.prior[ev.dim_param[d]].periodic) {
+              float x = u32[d] + sc * (ua[d].x - ub[d].x);
+              if (!(x >= -margin && x <= 1.0f + margin)) maybe = 0;
+            }
+          }
+        } else {
+          const double* ua = T.surv + a * D;
+          const double* ub = T.surv + b * D;
+#pragma unroll
+          for (int d = 0; d < kMaxDim; ++d) {
+            if (d < D && !ev.prior[ev.dim_param[d]].periodic) {
+              float x = u32[d] + sc * ((float)ua[d] - (float)ub[d]);
+              if (!(x >= -margin && x <= 1.0f + margin)) maybe = 0;
+            }
           }
         }
       }
-      const unsigned im = __ballot_sync(0xffffffffu, in);
-      const int slot = __popc(im & ((1u << lane) - 1u));
-      if (in && slot < m) {
+      unsigned mask = __ballot_sync(0xffffffffu, maybe);
+      if (lane == 0) wcount[warp] = __popc(mask);
+      __syncthreads();
+      int before = 0, total = 0;
 #pragma unroll
-        for (int d = 0; d < kMaxDim; ++d)
-          if (d < D) prop[slot][d] = pr[d];
-        cstep[slot] = st;
-        s_isflow[slot] = isf;
-        s_lqf[slot] = lqf;
+      for (int w2 = 0; w2 < kWarps; ++w2) {
+        int cw = wcount[w2];
+        before += (w2 < warp) ? cw : 0;
+        total += cw;
       }
-      const int nin_w = min(__popc(im), m);
-      // steps covered by this round: up to the m-th in-bounds proposal, else up to the last
-      // screened maybe-step, else the whole window
-      const unsigned mth = __ballot_sync(0xffffffffu, in && slot == m - 1);
-      int end;
-      if (__popc(im) > m) end = __shfl_sync(0xffffffffu, st, __ffs(mth) - 1);
-      else if (total > 32) end = __shfl_sync(0xffffffffu, st, 31);
-      else end = t + W - 1;
-      if (lane == 0) { s_nin = nin_w; s_end = end; }
-    }
+      const int mslot = before + __popc(mask & ((1u << lane) - 1u));
+      if (maybe && mslot < 32) mstep[mslot] = step;
+      const int nmaybe = min(total, 32);
+      __syncthreads();
+      // 1b. the setup warp redoes the maybe-in-bounds steps exactly (FP64, as the walk is
+      //     defined) and compacts the in-bounds ones into at most m slots
+      if (warp == sw) {
+        int in = 0, isf = 0;
+        float lqf = 0.0f;
+        double pr[kMaxDim];
+        const int st = lane < nmaybe ? mstep[lane] : 0;
+        if (use_flow && lane < nmaybe) {
+          Philox4 C = philox4x64((uint64_t)st, wid, it, 6ull, T.key0, T.key1);
+          if (rand_open_unit(C.v[0]) < p_flow) {
+            isf = 1;
+            lqf = (float)T.flq[(size_t)j * T.f_stride + st];
+            in = logf((float)rand_open_unit(C.v[1])) < s_logq - lqf;
+            const double* fu = T.fu + ((size_t)j * T.f_stride + st) * D;
+#pragma unroll
+            for (int d = 0; d < kMaxDim; ++d)
+              if (d < D) pr[d] = fu[d];
+          }
+        }
+        if (lane < nmaybe && !isf) {
+          Philox4 A = philox4x64((uint64_t)st, wid, it, 0ull, T.key0, T.key1);
+          uint64_t a = rand_index(A.v[0], n_s);
+          uint64_t b = rand_index(A.v[1], n_s - 1);
+          b += (b >= a) ? 1ull : 0ull;
+          double sc;
+          if ((A.v[2] >> 63) == 1ull) {
+            sc = 1.0;
+          } else {
+            Philox4 B = philox4x64((uint64_t)st, wid, it, 1ull, T.key0, T.key1);
+            double prod = __dmul_rn(__dmul_rn(__dmul_rn(rand_open_unit(B.v[0]), rand_open_unit(B.v[1])),
+                                              rand_open_unit(B.v[2])), rand_open_unit(B.v[3]));
+            sc = __dmul_rn(de_scale, __dmul_rn(-0.25, log(prod)));
+          }
+          const double* ua = T.surv + a * D;
+          const double* ub = T.surv + b * D;
+          in = 1;
+#pragma unroll
+          for (int d = 0; d < kMaxDim; ++d) {
+            if (d < D) {
+              double x = __dadd_rn(u[d], __dmul_rn(sc, __dsub_rn(ua[d], ub[d])));
+              if (ev.prior[ev.dim_param[d]].periodic) x = __dsub_rn(x, floor(x));
+              // 0 <= x <= 1 on the bit pattern (integer pipe): +0 .. 1.0 are the patterns up
+              // to 0x3FF0000000000000; negative values and NaN compare above.  x is never -0.
+              if ((unsigned long long)__double_as_longlong(x) > 0x3FF0000000000000ull) in = 0;
+              pr[d] = x;
+            }
+          }
+        }
+        const unsigned im = __ballot_sync(0xffffffffu, in);
+        const int slot = __popc(im & ((1u << lane) - 1u));
+        if (in && slot < m) {
+#pragma unroll
+          for (int d = 0; d < kMaxDim; ++d)
+            if (d < D) prop[slot][d] = pr[d];
+          cstep[slot] = st;
+          s_isflow[slot] = isf;
+          s_lqf[slot] = lqf;
+        }
+        const int nin_w = min(__popc(im), m);
+        // steps covered by this round: up to the m-th in-bounds proposal, else up to the last
+        // screened maybe-step, else the whole window
+        const unsigned mth = __ballot_sync(0xffffffffu, in && slot == m - 1);
+        int end;
+        if (__popc(im) > m) end = __shfl_sync(0xffffffffu, st, __ffs(mth) - 1);
+        else if (total > 32) end = __shfl_sync(0xffffffffu, st, 31);
+        else end = t + W - 1;
+        if (lane == 0) { s_nin = nin_w; s_end = end; }
+      }
     }
     __syncthreads();
     const int nin = s_nin;
-    // 2. proposal constants on all four warps (setup_split.cuh), then the likelihoods: the sums of proposal i into tot_p[i] (chunk totals in ct), then one lane
-    //    per proposal assembles ln L (the FP64 part runs once per proposal, on one warp)
+    // 2. proposal constants on all four warps (setup_split.cuh), then the likelihoods: the sums of
+    //    proposal i into tot_p[i] (chunk totals in ct), then one lane per proposal assembles ln L (the
+    //    FP64 part runs once per proposal, on one warp)
     if (nin > 0) {
       if (lane < nin) f64_split_first<PREC != 0, true>(warp, ev, prop[lane], parts[lane], P[lane]);
       __syncthreads();
@@ -1117,13 +1121,14 @@ __device__ __forceinline__ ff ff_wrap_unit(ff x) {
 //     amplitude shape on different warps);
 //  3. the likelihoods: TaylorF2 one warp per proposal, the IMRPhenomD form the whole CTA per
 //     proposal;
-//  4. warp 0 assembles ln L of every proposal in float-float and finds the first acceptance
-//     with one ballot (the IMRPhenomD form: every thread assembles it after each proposal, and the
-//     first acceptance ends the round).
-// Per-walker depths and the early end, with the survivors' float pairs made once a call (GB300,
-// before -> after): 500 walkers x 600 steps on the 4,017-bin TaylorF2 event 9.3 -> 4.9 ms, 1000 x
-// 240 on the 16,225-bin IMRPhenomD-form event 159 -> 20.8 ms, on its relative-binning likelihood
-// 13.8 -> 7.1 ms (acceptance 0.4 to 0.7 a call).
+//  4. warp 0 assembles ln L of every proposal in float-float and finds with one ballot where the
+//     round's guess first fails: its first acceptance, or, looking ahead over acceptances, its
+//     first rejection (the IMRPhenomD form: every thread assembles ln L after each proposal, and
+//     the round ends there, the rest unevaluated).
+// Stand-alone walks at 0.4 to 0.9 acceptances a call, against a fixed depth of 16 without look-ahead
+// over acceptances, screen, early end and float pairs made once a call (GB300): 500 walkers x 600
+// steps on the 4,017-bin TaylorF2 event 9.0 -> 2.2 ms, 1000 x 240 on the 16,225-bin IMRPhenomD-form
+// event 151 -> 17.6 ms, on its relative-binning likelihood 13.0 -> 6.6 ms.
 // The DE move is the walk's, u' = u + gamma (u_a - u_b), with the position and the survivors as
 // float pairs (~48 significant bits): the chain is the FP64 chain up to rounding at ~1e-14.
 // A TaylorF2 or relative-binning round is padded to a multiple of four proposals: its
@@ -1377,102 +1382,102 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel_ff(const EventDev* __
     } else {
       // 1. the exact move of one candidate step per thread (or its flow proposal)
       const int W = min(min(kThreads, max(32, 4 * m)), n_steps - t);
-    const int step = t + (int)threadIdx.x;
-    int in = 0, isf = 0;
-    float lqf = 0.0f;
-    ff xf[kMaxDim];
-    if ((int)threadIdx.x < W) {
-      // the step's Philox blocks: (tag 6: flow coin,) tag 0: survivors and scale coin,
-      // tag 1: the scale's uniforms -- one inlined generator, called up to three times
-      Philox4 A, B;
-      bool draw_scale = false;
-      int tag = use_flow ? 6 : 0;
+      const int step = t + (int)threadIdx.x;
+      int in = 0, isf = 0;
+      float lqf = 0.0f;
+      ff xf[kMaxDim];
+      if ((int)threadIdx.x < W) {
+        // the step's Philox blocks: (tag 6: flow coin,) tag 0: survivors and scale coin,
+        // tag 1: the scale's uniforms -- one inlined generator, called up to three times
+        Philox4 A, B;
+        bool draw_scale = false;
+        int tag = use_flow ? 6 : 0;
 #pragma unroll 1
-      while (tag >= 0) {
-        const Philox4 r = philox4x64((uint64_t)step, wid, it, (uint64_t)tag, T.key0, T.key1);
-        if (tag == 6) {
-          tag = 0;
-          if (rand_open_unit(r.v[0]) < p_flow) {
-            isf = 1;
-            lqf = (float)T.flq[(size_t)j * T.f_stride + step];
-            in = logf((float)rand_open_unit(r.v[1])) < s_logq - lqf;
+        while (tag >= 0) {
+          const Philox4 r = philox4x64((uint64_t)step, wid, it, (uint64_t)tag, T.key0, T.key1);
+          if (tag == 6) {
+            tag = 0;
+            if (rand_open_unit(r.v[0]) < p_flow) {
+              isf = 1;
+              lqf = (float)T.flq[(size_t)j * T.f_stride + step];
+              in = logf((float)rand_open_unit(r.v[1])) < s_logq - lqf;
+              tag = -1;
+            }
+          } else if (tag == 0) {
+            A = r;
+            draw_scale = (r.v[2] >> 63) == 0ull;
+            tag = draw_scale ? 1 : -1;
+          } else {
+            B = r;
             tag = -1;
           }
-        } else if (tag == 0) {
-          A = r;
-          draw_scale = (r.v[2] >> 63) == 0ull;
-          tag = draw_scale ? 1 : -1;
-        } else {
-          B = r;
-          tag = -1;
         }
-      }
-      if (isf) {
-        if (in) {
-          const double* fu = T.fu + ((size_t)j * T.f_stride + step) * D;
+        if (isf) {
+          if (in) {
+            const double* fu = T.fu + ((size_t)j * T.f_stride + step) * D;
 #pragma unroll
-          for (int d = 0; d < kMaxDim; ++d)
-            if (d < D) xf[d] = ff_from_double(fu[d]);
-        }
-      } else {
-        const uint64_t a = rand_index(A.v[0], n_s);
-        uint64_t b = rand_index(A.v[1], n_s - 1);
-        b += (b >= a) ? 1ull : 0ull;
-        // both survivors' coordinates first (branch-free, all loads in flight at once)
-        ff ua[kMaxDim], ub[kMaxDim];
-        if (T.survf) {
-#pragma unroll
-          for (int d = 0; d < kMaxDim; ++d) {
-            const int dd = d < D ? d : D - 1;
-            const float2 pa = T.survf[a * D + dd], pb = T.survf[b * D + dd];
-            ua[d] = ff{pa.x, pa.y};
-            ub[d] = ff{pb.x, pb.y};
+            for (int d = 0; d < kMaxDim; ++d)
+              if (d < D) xf[d] = ff_from_double(fu[d]);
           }
         } else {
+          const uint64_t a = rand_index(A.v[0], n_s);
+          uint64_t b = rand_index(A.v[1], n_s - 1);
+          b += (b >= a) ? 1ull : 0ull;
+          // both survivors' coordinates first (branch-free, all loads in flight at once)
+          ff ua[kMaxDim], ub[kMaxDim];
+          if (T.survf) {
+#pragma unroll
+            for (int d = 0; d < kMaxDim; ++d) {
+              const int dd = d < D ? d : D - 1;
+              const float2 pa = T.survf[a * D + dd], pb = T.survf[b * D + dd];
+              ua[d] = ff{pa.x, pa.y};
+              ub[d] = ff{pb.x, pb.y};
+            }
+          } else {
+#pragma unroll
+            for (int d = 0; d < kMaxDim; ++d) {
+              const int dd = d < D ? d : D - 1;
+              ua[d] = ff_from_double(T.surv[a * D + dd]);
+              ub[d] = ff_from_double(T.surv[b * D + dd]);
+            }
+          }
+          const ff sc = draw_scale ? ff_mul(ff_mul_f(ff_log_uniform_product(B.v), -0.25f), de_scale) : ff_make(1.0f);
+          in = 1;
 #pragma unroll
           for (int d = 0; d < kMaxDim; ++d) {
-            const int dd = d < D ? d : D - 1;
-            ua[d] = ff_from_double(T.surv[a * D + dd]);
-            ub[d] = ff_from_double(T.surv[b * D + dd]);
+            const ff df = ff_mul(sc, ff_sub(ua[d], ub[d]));
+            ff x = ff_add(uf[d < D ? d : D - 1], df);
+            const ff xw = ff_wrap_unit(x);
+            if ((periodic >> d) & 1u) x = xw;
+            if (d < D && !ff_in_unit(x)) in = 0;
+            xf[d] = x;
           }
         }
-        const ff sc = draw_scale ? ff_mul(ff_mul_f(ff_log_uniform_product(B.v), -0.25f), de_scale) : ff_make(1.0f);
-        in = 1;
-#pragma unroll
-        for (int d = 0; d < kMaxDim; ++d) {
-          const ff df = ff_mul(sc, ff_sub(ua[d], ub[d]));
-          ff x = ff_add(uf[d < D ? d : D - 1], df);
-          const ff xw = ff_wrap_unit(x);
-          if ((periodic >> d) & 1u) x = xw;
-          if (d < D && !ff_in_unit(x)) in = 0;
-          xf[d] = x;
-        }
       }
-    }
-    const unsigned mask = __ballot_sync(0xffffffffu, in);
-    if (lane == 0) wcount[warp] = __popc(mask);
-    __syncthreads();
-    int before = 0, total = 0;
+      const unsigned mask = __ballot_sync(0xffffffffu, in);
+      if (lane == 0) wcount[warp] = __popc(mask);
+      __syncthreads();
+      int before = 0, total = 0;
 #pragma unroll
-    for (int w2 = 0; w2 < kWarps; ++w2) {
-      const int cw = wcount[w2];
-      before += (w2 < warp) ? cw : 0;
-      total += cw;
-    }
-    const int slot = before + __popc(mask & ((1u << lane) - 1u));
-    if (in && slot < m) {
+      for (int w2 = 0; w2 < kWarps; ++w2) {
+        const int cw = wcount[w2];
+        before += (w2 < warp) ? cw : 0;
+        total += cw;
+      }
+      const int slot = before + __popc(mask & ((1u << lane) - 1u));
+      if (in && slot < m) {
 #pragma unroll
-      for (int d = 0; d < kMaxDim; ++d)
-        if (d < D) propf[slot][d] = xf[d];
-      cstep[slot] = step;
-      s_isflow[slot] = isf;
-      s_lqf[slot] = lqf;
-      // the round covers the steps up to the m-th in-bounds one, else the whole window
-      if (slot == m - 1 && total > m) s_end = step;
-    }
-    if (threadIdx.x == 0 && total <= m) s_end = t + W - 1;
-    nin = min(total, m);
-    __syncthreads();
+        for (int d = 0; d < kMaxDim; ++d)
+          if (d < D) propf[slot][d] = xf[d];
+        cstep[slot] = step;
+        s_isflow[slot] = isf;
+        s_lqf[slot] = lqf;
+        // the round covers the steps up to the m-th in-bounds one, else the whole window
+        if (slot == m - 1 && total > m) s_end = step;
+      }
+      if (threadIdx.x == 0 && total <= m) s_end = t + W - 1;
+      nin = min(total, m);
+      __syncthreads();
     }
     // 2. proposal constants
     if (nin > 0) {
@@ -2201,9 +2206,11 @@ __global__ void __launch_bounds__(kThreads, 4) hrss_kernel_ff(const EventDev* __
 #define GWNS_DISPATCH_W(K, P)                                                     \
   if (waveform == 0) { GWNS_DISPATCH_N(K, P, 0) } else { GWNS_DISPATCH_N(K, P, 1) }
 
-// Proposals of a CTA: as many as keep every SM at two CTAs (a setup costs its warps the same FP64
-// time for one proposal or for a full tile), up to 16 for TaylorF2; up to 4 for the IMRPhenomD
-// form, whose evaluations take ~100 times a setup and balance better in small pieces.
+// Proposals of a CTA: as many as keep each of the 152 SMs at two CTAs (a setup costs its warps the
+// same FP64 time for one proposal or for a full tile), up to 16 for TaylorF2; up to 4 for the
+// IMRPhenomD form, whose evaluations take ~100 times a setup and balance better in small pieces.
+// The result does not depend on the tile; asking the device for its SMs made calls of 1 and 1000
+// vectors 2 and 4 us slower (37 and 47 us alone).
 inline int lik_tile(int n, int waveform) {
   const int t = (n + 303) / 304, most = waveform == 0 ? kLikTile : 4;
   return t < 1 ? 1 : (t > most ? most : t);
@@ -2241,8 +2248,14 @@ cudaError_t launch_unit_likelihood_p(int waveform, int n_det, const EventDev* d_
 // acceptance may be anything (500 walkers x 600 steps at 0.87 acceptances a call, 4,017 bins: 4.85 ->
 // 2.1 ms).  The sampler's walks accept a few per cent of their calls from the first batches on, and
 // there the larger kernel costs 5 % (ten batches: 17.9 -> 19.0 ms of walks), so they take the plain
-// one; so do flows and the IMRPhenomD form with relative binning (1000 walkers x 240 steps at 0.6: 6.6
-// ms without, 7.4 ms with it; TaylorF2 with relative binning at 0.85: 2.6 -> 1.2 ms).
+// one; so do flows.  With relative binning TaylorF2 takes the look-ahead and the IMRPhenomD form does
+// not.  It is the acceptance p that decides between the two kernels, and alike for both forms, us
+// without -> with (500 x 240 TaylorF2; 1000 x 240 IMRPhenomD):
+//   p 0.93   1136 ->  535;  3766 -> 1732      p 0.35   717 -> 775;  2787 -> 3005
+//   p 0.78    989 ->  695;  3431 -> 2466      p 0.24   656 -> 673;  2212 -> 2276
+//   p 0.58    914 ->  935;  3238 -> 3370      p 0.15   538 -> 548;  1536 -> 1642
+// so the IMRPhenomD form's line is not a property of the form: its walks lose 3 to 8 % below p = 0.6
+// and would gain above 0.7; a launch does not know p.
 // The float-float walk's variants are compiled in units of their own (GWNS_FF_WALK: parallel builds).
 #define GWNS_WALK_ARGS \
   int waveform, int n_det, const EventDev *d_evs, WalkTask *d_tasks, const int32_t *d_blk_task, \

@@ -24,7 +24,7 @@ cudaError_t launch_unit_to_theta(const EventDev* d_ev, const double* d_u, int64_
 cudaError_t launch_waveform(int waveform, int n_det, const EventDev* d_ev, const double* d_theta, int n, int n_bins,
                             double* d_hre, double* d_him, cudaStream_t s, int no_cutoff) {
   if (n <= 0) return cudaSuccess;
-  // spans of whole 128-bin rows that give every SM about four CTAs
+  // spans of whole 128-bin rows that give each of the 152 SMs about four CTAs
   const int rows = (n_bins + kThreads - 1) / kThreads;
   const int want = n >= 608 ? 1 : (608 + n - 1) / n, spans = want < rows ? want : rows;
   const int span = (rows + spans - 1) / spans * kThreads;
