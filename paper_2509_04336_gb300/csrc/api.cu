@@ -471,6 +471,11 @@ extern "C" int ns_likelihood_batch(ns_handle* h, int event, const double* theta,
   return e == cudaSuccess ? NS_OK : cuda_fail(h, e, "likelihood launch");
 }
 
+// Bytes of the float pairs that a stand-alone walk keeps in the handle's scratch: room for 700,000
+// points of eleven coordinates, a hundred times the largest live set, so that the scratch of a
+// handle does not grow with whatever array a caller draws its differences from.
+static const size_t kWalkPairsMax = (size_t)64 << 20;
+
 extern "C" int ns_walk_batch(ns_handle* h, int event, const double* live_u, int n_live_pts, const double* u0,
                              const double* lnl0, double lnl_star, int n, int n_steps, int64_t iteration,
                              int64_t walker_offset, double* u_out, double* lnl_out, int32_t* n_accept,
@@ -512,16 +517,18 @@ extern "C" int ns_walk_batch(ns_handle* h, int event, const double* live_u, int 
     return cuda_fail(h, e, "status reset");
   int fr = flow_attach(h, event, T, n, n_steps, &h->scratch_flow, s);
   if (fr) return fr;
-  // one task slot of the handle, block -> (event, walker) maps, the survivors as float pairs
+  // one task slot of the handle, block -> (event, walker) maps, the survivors as float pairs (not of
+  // arrays beyond kWalkPairsMax: the walks then convert the doubles that they read, to the same pairs)
   const size_t nu = (size_t)n * D, ns_ = (size_t)n_live_pts * D;
   const size_t task_b = (sizeof(WalkTask) + 255) / 256 * 256, map_b = (sizeof(int32_t) * 2 * (size_t)n + 255) / 256 * 256;
-  int r = ensure_scratch(h, h->scratch_map, task_b + map_b + sizeof(float2) * ns_);
+  const size_t n_pairs = sizeof(float2) * ns_ <= kWalkPairsMax ? ns_ : 0;
+  int r = ensure_scratch(h, h->scratch_map, task_b + map_b + sizeof(float2) * n_pairs);
   if (r) return r;
   WalkTask* d_task = (WalkTask*)h->scratch_map.ptr;
   int32_t* d_be = (int32_t*)((char*)h->scratch_map.ptr + task_b);
   int32_t* d_bl = d_be + n;
   float2* d_survf = (float2*)((char*)h->scratch_map.ptr + task_b + map_b);
-  T.survf = d_survf;
+  T.survf = n_pairs ? d_survf : nullptr;
   int32_t* clear = flow ? nullptr : h->d_status + 1;
   if (ptr_kind == NS_PTR_HOST) {
     if (!finite_array(live_u, (int)ns_) || !finite_array(u0, (int)nu)) return set_error(h, NS_ENONFINITE, "u not finite");
@@ -541,7 +548,7 @@ extern "C" int ns_walk_batch(ns_handle* h, int event, const double* live_u, int 
         (e = cudaMemcpyAsync(d_u0, u0, sizeof(double) * nu, cudaMemcpyHostToDevice, s)) ||
         (e = cudaMemcpyAsync(d_l0, lnl0, sizeof(double) * n, cudaMemcpyHostToDevice, s)))
       return cuda_fail(h, e, "H2D walk inputs");
-    if ((e = launch_walk_prepare(T, d_task, d_be, d_bl, d_survf, clear, ns_, s)) != cudaSuccess ||
+    if ((e = launch_walk_prepare(T, d_task, d_be, d_bl, d_survf, clear, n_pairs, s)) != cudaSuccess ||
         (e = launch_walk(h->precision, h->waveform, E.n_det, h->d_events, d_task, d_be, d_bl, n, s, walk_extras(h, event), true)) != cudaSuccess)
       return cuda_fail(h, e, "walk launch");
     if ((e = cudaMemcpyAsync(u_out, d_uo, sizeof(double) * nu, cudaMemcpyDeviceToHost, s)) ||
@@ -555,7 +562,7 @@ extern "C" int ns_walk_batch(ns_handle* h, int event, const double* live_u, int 
     return NS_OK;
   }
   T.surv = live_u; T.u0 = u0; T.lnl0 = lnl0; T.u_out = u_out; T.lnl_out = lnl_out; T.n_acc = n_accept; T.n_like = n_like;
-  if ((e = launch_walk_prepare(T, d_task, d_be, d_bl, d_survf, clear, ns_, s)) != cudaSuccess)
+  if ((e = launch_walk_prepare(T, d_task, d_be, d_bl, d_survf, clear, n_pairs, s)) != cudaSuccess)
     return cuda_fail(h, e, "walk task launch");
   e = launch_walk(h->precision, h->waveform, E.n_det, h->d_events, d_task, d_be, d_bl, n, s, walk_extras(h, event), true);
   return e == cudaSuccess ? NS_OK : cuda_fail(h, e, "walk launch");
