@@ -678,26 +678,15 @@ __global__ void __launch_bounds__(kThreads) waveform_kernel(const EventDev* __re
 // sampler's walks, whose batch rule knows p (their own estimates, noisier, gained nothing).  Any choice gives the same
 // chain.  pad4: rounds of a warp per proposal, padded to a multiple of four.  CH: compiled with the
 // look-ahead over acceptances.
-//   lead: how far acceptances must lead before a round looks ahead over them.  Without one, a
-// walker whose first call was accepted bet its next round on acceptances and at p = 0.15 lost it
-// to the first rejection, where a round over rejections would have resolved several calls: short
-// walks of few acceptances, whose slowest walker had met this once or twice, took up to 1.2 times
-// as long as at the fixed depth.  Lead 0 -> 1, in us (fixed depth): 50 walkers x 120 steps, TaylorF2
-// float-float, p 0.16, 228 -> 208 (214); 500 x 80, FP64 phase, p 0.05, 377 -> 335 (331); 300 x 60,
-// 16,225 bins, FP64 phase, p 0.02, 5239 -> 4337 (4995); 50 x 40, relative binning, p 0.04, 161 -> 141
-// (145).  At p 0.6 to 0.9, 500 x 600 float-float 2229 -> 2243, 500 x 240 FP64 phase 2743 -> 2737, 500 x
-// 120 relative binning 440 -> 488 (958).  No lead where a lost round was cheap and nothing was lost:
-// FP64 walks (fixed depth 4; a lead costs them 3 % at p 0.7) and the float-float IMRPhenomD form
-// (a round ends at its first wrong guess; 3 to 6 % at p 0.8).
 struct Round {
   int depth;
   bool chain;
 };
 template <bool CH>
-__device__ __forceinline__ Round next_round(const WalkTask& T, bool pad4, int lead, int n_acc, int n_like) {
+__device__ __forceinline__ Round next_round(const WalkTask& T, bool pad4, int n_acc, int n_like) {
   Round r;
   r.depth = T.spec < 1 ? 1 : (T.spec > kSpecMax ? kSpecMax : T.spec);
-  r.chain = CH && T.spec_cap > 0 && 2 * n_acc > n_like + lead;
+  r.chain = CH && T.spec_cap > 0 && 2 * n_acc > n_like;
   if (T.spec_cap > 0) {
     const int ends = r.chain ? n_like - n_acc : n_acc;
     r.depth = (int)(1.4f * ((float)n_like + (float)r.depth) / ((float)ends + 1.4f) + 0.5f);
@@ -794,7 +783,7 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel(const EventDev* __res
   const int sw = s_setup_warp;
   const bool use_flow = !CH && T.flow != nullptr && T.p_flow > 0.0;
   const double p_flow = T.p_flow;
-  Round rd = next_round<CH>(T, false, PREC == 0 ? 0 : 1, 0, 0);
+  Round rd = next_round<CH>(T, false, 0, 0);
   if (use_flow) {
     const float lq = flow_logq_cta(*T.flow, u, fscr);
     if (threadIdx.x == 0) s_logq = lq;
@@ -1067,7 +1056,7 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel(const EventDev* __res
         if (T.status && rank == 0) atomicOr(T.status, 1);
       }
       s_next = nxt;
-      s_round = next_round<CH>(T, false, PREC == 0 ? 0 : 1, n_acc, n_like);
+      s_round = next_round<CH>(T, false, n_acc, n_like);
     }
     __syncthreads();
     t = s_next;
@@ -1208,7 +1197,7 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel_ff(const EventDev* __
   const int sw = s_setup_warp;
   const bool use_flow = XF && T.flow != nullptr && T.p_flow > 0.0;
   const double p_flow = T.p_flow;
-  Round rd = next_round<CH>(T, WF == 0 || (X >= 1 && ev.rb_nb > 0), WF == 0 ? 1 : 0, 0, 0);
+  Round rd = next_round<CH>(T, WF == 0 || (X >= 1 && ev.rb_nb > 0), 0, 0);
   if (use_flow) {
     const float lq = flow_logq_cta(*T.flow, u, fscr);
     if (threadIdx.x == 0) s_logq = lq;
@@ -1628,7 +1617,7 @@ __global__ void __launch_bounds__(kThreads, 4) walk_kernel_ff(const EventDev* __
           if (T.status) atomicOr(T.status, 1);
         }
         s_next = nxt;
-        s_round = next_round<CH>(T, WF == 0 || (X >= 1 && ev.rb_nb > 0), WF == 0 ? 1 : 0, n_acc, n_like);
+        s_round = next_round<CH>(T, WF == 0 || (X >= 1 && ev.rb_nb > 0), n_acc, n_like);
       }
     }
     __syncthreads();
