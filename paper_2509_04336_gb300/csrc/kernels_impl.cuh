@@ -675,9 +675,12 @@ __global__ void __launch_bounds__(kThreads) waveform_kernel(const EventDev* __re
 // 1.4 / (1 - p), with the task's depth as the first estimate, worth 1.4 outcomes of the other kind.
 // A stand-alone walk has no batch before it: a fixed depth of 16 dropped 9 of 10 evaluations at
 // p = 0.6.  spec_cap 0 keeps the task's depth, over rejections: a depth fixed by the user, and the
-// sampler's walks, whose batch rule knows p (their own estimates, noisier, gained nothing).  Any choice gives the same
-// chain.  pad4: rounds of a warp per proposal, padded to a multiple of four.  CH: compiled with the
-// look-ahead over acceptances.
+// sampler's walks, whose batch rule knows p (their own estimates, noisier, gained nothing).  Any
+// choice gives the same chain.  Asking acceptances to lead by one call before a round looks ahead
+// over them spares a walker whose first call was accepted by luck: 4 to 13 % of a 60- or 200-step
+// walk at p below 0.2, but it costs 4 to 17 % above 0.75, and against the fixed depth walks of low p
+// lose 2 % at most without it (means of four walks each).  pad4: rounds of a warp per proposal,
+// padded to a multiple of four.  CH: compiled with the look-ahead over acceptances.
 struct Round {
   int depth;
   bool chain;
@@ -2240,10 +2243,10 @@ cudaError_t launch_unit_likelihood_p(int waveform, int n_det, const EventDev* d_
 // one; so do flows.  With relative binning TaylorF2 takes the look-ahead and the IMRPhenomD form does
 // not.  It is the acceptance p that decides between the two kernels, and alike for both forms, us
 // without -> with (500 x 240 TaylorF2; 1000 x 240 IMRPhenomD):
-//   p 0.93   1136 ->  535;  3766 -> 1732      p 0.35   717 -> 775;  2787 -> 3005
-//   p 0.78    989 ->  695;  3431 -> 2466      p 0.24   656 -> 673;  2212 -> 2276
-//   p 0.58    914 ->  935;  3238 -> 3370      p 0.15   538 -> 548;  1536 -> 1642
-// so the IMRPhenomD form's line is not a property of the form: its walks lose 3 to 8 % below p = 0.6
+//   p 0.93   1057 ->  458;  3807 -> 1585      p 0.35   708 -> 782;  2772 -> 3071
+//   p 0.78    957 ->  644;  3439 -> 2315      p 0.24   648 -> 693;  2220 -> 2347
+//   p 0.58    876 ->  835;  3199 -> 3234      p 0.15   535 -> 560;  1547 -> 1658
+// so the IMRPhenomD form's line is not a property of the form: its walks lose 1 to 10 % below p = 0.6
 // and would gain above 0.7; a launch does not know p.
 // The float-float walk's variants are compiled in units of their own (GWNS_FF_WALK: parallel builds).
 #define GWNS_WALK_ARGS \
